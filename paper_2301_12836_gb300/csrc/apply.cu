@@ -340,6 +340,10 @@ __global__ void __launch_bounds__(NTH) k_strided_raw(FftPlan p, const typename c
     strided_tile<DIR, GenericFFT>(src, dst, p, tw, a, blockIdx.x * a.TX, sa, sb);
 }
 
+}  // namespace lsm
+#include "apply_fx.cuh"
+namespace lsm {
+
 // four-step strided pass: step 1 loads straight from global memory, the last step stores straight
 // to global memory; one shared-memory exchange in between.  Block = TX * TPL threads, line l = lx.
 template <typename T, int DIR, int A, int B, int TX>
@@ -1366,32 +1370,44 @@ static void strided_cfg(int L, int ncomp, int& TX, int& threads, size_t& sm, int
     }
 }
 
-// forward x FFT of the contrast source rows: w2 [3][ez][ey][ex] -> w1 [3][ez][ey][Lx]
+// forward x FFT of nrows rows of in_count elements, zero-padded to Lx: src_sel -> dst_sel [nrows][Lx]
 template <typename T>
-static void launch_xfwd(const Dims& d, const ApplySys<T>* sys, int nsys, const Plans& pl, cudaStream_t st, int v = 0) {
+static void launch_xrows(const Dims& d, const ApplySys<T>* sys, int nsys, const Plans& pl, int src_sel, int dst_sel,
+                         long long nrows, int in_count, cudaStream_t st, int v = 0) {
     typedef typename cplx_of<T>::type C;
-    if (!fourstep_prunable(d.Lx, d.ex, 0)) v = 1;
-    const long long nrows = 3LL * d.ez * d.ey;
+    if (!fourstep_prunable(d.Lx, in_count, 0)) v = 1;
     with_engine<std::is_same<T, dfloat>::value>(d.Lx, [&](auto eng) {
         using F = decltype(eng);
-        if constexpr (F::INPLACE && F::A_ == F::B_) {
+        if constexpr (F::INPLACE && std::is_same<T, double>::value) {
+            constexpr int A = F::A_, B = F::B_, LPB = 128 / F::TPL;
+            const size_t sm = (size_t)LPB * B * (A + 1) * sizeof(fxc);
+            smem_attr((const void*)k4_rows_fx<A, B, LPB>, sm);
+            k4_rows_fx<A, B, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * F::TPL, sm, st>>>(
+                pl.fxx, sys, src_sel, dst_sel, nrows, in_count, fx_bits(A * B, in_count, A / 2 + 1, B));
+        } else if constexpr (F::INPLACE && F::A_ == F::B_) {
             constexpr int A = F::A_, LPB = sizeof(T) == 4 ? 16 : 8;
-            k4_rows_w<T, A, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * A, 0, st>>>((const C*)pl.twx, sys, 3, 2, nrows,
-                                                                                   d.ex);
+            k4_rows_w<T, A, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * A, 0, st>>>((const C*)pl.twx, sys, src_sel, dst_sel,
+                                                                                   nrows, in_count);
         } else if constexpr (F::INPLACE) {
             constexpr int A = F::A_, B = F::B_, NL = sizeof(T) == 4 ? 8 : 12;
             const size_t sm = (size_t)A * B * (NL + 1) * sizeof(C);
             smem_attr((const void*)k4_rows<T, -1, A, B, NL>, sm);
             k4_rows<T, -1, A, B, NL><<<dim3(cdiv(nrows, NL), nsys), NL * F::TPL, sm, st>>>(
-                (const C*)pl.twx, sys, 3, 2, nrows, d.ex, 0, d.Lx, 0);
+                (const C*)pl.twx, sys, src_sel, dst_sel, nrows, in_count, 0, d.Lx, 0);
         } else {
             const int NL = generic_rows_nl<T>(d.Lx, v == 2);
             const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(C);
             smem_attr((const void*)k_rows<T, -1>, sm);
-            k_rows<T, -1><<<dim3(cdiv(nrows, NL), nsys), NTH, sm, st>>>(pl.px, (const C*)pl.twx, sys, 3, 2, nrows, NL,
-                                                                         d.ex, 0, d.Lx, 0);
+            k_rows<T, -1><<<dim3(cdiv(nrows, NL), nsys), NTH, sm, st>>>(pl.px, (const C*)pl.twx, sys, src_sel, dst_sel, nrows,
+                                                                         NL, in_count, 0, d.Lx, 0);
         }
     }, v);
+}
+
+// forward x FFT of the contrast source rows: w2 [3][ez][ey][ex] -> w1 [3][ez][ey][Lx]
+template <typename T>
+static void launch_xfwd(const Dims& d, const ApplySys<T>* sys, int nsys, const Plans& pl, cudaStream_t st, int v = 0) {
+    launch_xrows<T>(d, sys, nsys, pl, 3, 2, 3LL * d.ez * d.ey, d.ex, st, v);
 }
 
 // xoff: padded-grid index of model node 0 (1 when the convolved source lives on the extended nodes)
@@ -1404,7 +1420,13 @@ static void launch_fftx_out(const Dims& d, const ApplySys<T>* sys, int nsys, con
     typedef typename cplx_of<T>::type C;
     with_engine<std::is_same<T, dfloat>::value>(d.Lx, [&](auto eng) {
         using F = decltype(eng);
-        if constexpr (F::INPLACE && F::A_ == F::B_) {
+        if constexpr (F::INPLACE && std::is_same<T, double>::value) {
+            constexpr int A = F::A_, B = F::B_, LPB = 128 / F::TPL;
+            const size_t sm = (size_t)LPB * B * (A + 1) * sizeof(fxc);
+            smem_attr((const void*)k4_xout_fx<A, B, LPB>, sm);
+            k4_xout_fx<A, B, LPB><<<dim3(cdiv(3LL * d.nz * d.ny, LPB), nsys), LPB * F::TPL, sm, st>>>(
+                d, sys, pl.fxx, xoff, fx_bits(A * B, A * B, A, B));
+        } else if constexpr (F::INPLACE && F::A_ == F::B_) {
             constexpr int A = F::A_, LPB = sizeof(T) == 4 ? 16 : 8;
             const long long nrows = 3LL * d.nz * d.ny;
             if constexpr (std::is_same<T, float>::value) {
@@ -1441,8 +1463,8 @@ static void launch_fftx_out(const Dims& d, const ApplySys<T>* sys, int nsys, con
 // Plain FFT of lines of length L along a strided axis: a.ncomp components per system, lines along
 // x (a.nlines of them), `outer` line groups (blockIdx.y) per component.
 template <typename T, int DIR>
-static void launch_strided(int L, const FftPlan& p, const void* tw, StridedArgs a, int outer, const ApplySys<T>* sys,
-                           int nsys, cudaStream_t st, int v = 0) {
+static void launch_strided(int L, const FftPlan& p, const void* tw, const int4* fxtw, StridedArgs a, int outer,
+                           const ApplySys<T>* sys, int nsys, cudaStream_t st, int v = 0) {
     typedef typename cplx_of<T>::type C;
     if (!fourstep_prunable(L, DIR < 0 ? a.in_off + a.in_count : 0, DIR > 0 ? a.out_off + a.out_count : 0)) v = 1;
     with_engine<std::is_same<T, dfloat>::value>(L, [&](auto eng) {
@@ -1450,7 +1472,12 @@ static void launch_strided(int L, const FftPlan& p, const void* tw, StridedArgs 
         int th;
         size_t sm;
         strided_cfg<T, F>(L, 1, a.TX, th, sm, v == 2);
-        if constexpr (F::INPLACE) {
+        if constexpr (F::INPLACE && std::is_same<T, double>::value) {
+            constexpr int A = F::A_, B = F::B_, TXC = 8;
+            smem_attr((const void*)k4_strided_fx<DIR, A, B, TXC>, sm);
+            k4_strided_fx<DIR, A, B, TXC><<<dim3(cdiv(a.nlines, TXC), outer, a.ncomp * nsys), th, sm, st>>>(
+                fxtw, a, sys, fx_bits(L, a.in_count, DIR < 0 ? A / 2 + 1 : A, B));
+        } else if constexpr (F::INPLACE) {
             constexpr int A = F::A_, B = F::B_, TXC = sizeof(T) == 4 ? 16 : 8;
             smem_attr((const void*)k4_strided<T, DIR, A, B, TXC>, sm);
             k4_strided<T, DIR, A, B, TXC><<<dim3(cdiv(a.nlines, a.TX), outer, a.ncomp * nsys), th, sm, st>>>((const C*)tw, a, sys);
@@ -1472,7 +1499,7 @@ static void launch_ypass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
     a.src_es = d.Lx; a.src_os1 = (long long)in_count * d.Lx; a.src_os2 = (long long)planes * in_count * d.Lx;
     a.dst_es = d.Lx; a.dst_os1 = (long long)out_count * d.Lx; a.dst_os2 = (long long)planes * out_count * d.Lx;
     a.ncomp = ncomp; a.src_sel = src_sel; a.dst_sel = dst_sel;
-    launch_strided<T, DIR>(d.Ly, pl.py, pl.twy, a, planes, sys, nsys, st, v);
+    launch_strided<T, DIR>(d.Ly, pl.py, pl.twy, pl.fxy, a, planes, sys, nsys, st, v);
 }
 
 // plain z pass: src [ncomp][in_count][Ly][Lx] (sel) -> dst [ncomp][out_count][Ly][Lx] (sel)
@@ -1486,7 +1513,7 @@ static void launch_zplain(const Dims& d, const ApplySys<T>* sys, int nsys, const
     a.src_es = plane; a.src_os1 = d.Lx; a.src_os2 = (long long)in_count * plane;
     a.dst_es = plane; a.dst_os1 = d.Lx; a.dst_os2 = (long long)out_count * plane;
     a.ncomp = ncomp; a.src_sel = src_sel; a.dst_sel = dst_sel;
-    launch_strided<T, DIR>(d.Lz, pl.pz, pl.twz, a, d.Ly, sys, nsys, st);
+    launch_strided<T, DIR>(d.Lz, pl.pz, pl.twz, pl.fxz, a, d.Ly, sys, nsys, st);
 }
 
 // schedule variant v: 0 default (register-resident kernel for FP32 and L = A * A), 1 / 2 generic
@@ -1519,7 +1546,15 @@ static void launch_zpass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
             return;
           }
         }
-        if constexpr (F::INPLACE) {
+        if constexpr (F::INPLACE && std::is_same<T, double>::value) {
+            constexpr int A = F::A_, B = F::B_, TXC = F::TPL < 8 ? 16 : 4, NL = 3 * TXC;
+            constexpr int YB = B * fft4_ystride<A, fxc>(NL);
+            const size_t smf = (size_t)(YB > A * B * NL ? YB : A * B * NL) * sizeof(fxc) + (size_t)A * B * TXC * sizeof(int);
+            smem_attr((const void*)k4_fftz_green_fx<CONJ, A, B, TXC>, smf);
+            k4_fftz_green_fx<CONJ, A, B, TXC><<<dim3(cdiv(d.Lx, TXC) * nsys, d.Ly, 1), NL * F::TPL, smf, st>>>(
+                d, pl.fxz, sys, nsys, in_count, in_off, out_count, out_off, src_sel, dst_sel, fx_bits(A * B, in_count, A / 2 + 1, B),
+                fx_bits(A * B, A * B, A, B));
+        } else if constexpr (F::INPLACE) {
             constexpr int A = F::A_, B = F::B_, TXC = 4;
             smem_attr((const void*)k4_fftz_green<T, CONJ, A, B, TXC>, sm);
             k4_fftz_green<T, CONJ, A, B, TXC><<<dim3(cdiv(d.Lx, TXC), d.Ly, 1), th, sm, st>>>(
@@ -1624,29 +1659,7 @@ static cudaError_t launch_apply_h(const Medium& m, const Plans& pl, const ApplyS
     ktimer_mark(tm, 0, f32, st, 1);
     // 2. forward x FFT of the 9 planes: w1 -> w2 [9][nz][ny][Lx]
     ktimer_mark(tm, 1, f32, st, 0);
-    {
-        const long long nrows = 9LL * d.nz * d.ny;
-        with_engine<std::is_same<T, dfloat>::value>(d.Lx, [&](auto eng) {
-            using F = decltype(eng);
-            if constexpr (F::INPLACE && F::A_ == F::B_) {
-                constexpr int A = F::A_, LPB = sizeof(T) == 4 ? 16 : 8;
-                k4_rows_w<T, A, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * A, 0, st>>>((const C*)pl.twx, sys, 2, 3,
-                                                                                       nrows, d.nx);
-            } else if constexpr (F::INPLACE) {
-                constexpr int A = F::A_, B = F::B_, NL = sizeof(T) == 4 ? 8 : 12;
-                const size_t sm = (size_t)A * B * (NL + 1) * sizeof(C);
-                smem_attr((const void*)k4_rows<T, -1, A, B, NL>, sm);
-                k4_rows<T, -1, A, B, NL><<<dim3(cdiv(nrows, NL), nsys), NL * F::TPL, sm, st>>>(
-                    (const C*)pl.twx, sys, 2, 3, nrows, d.nx, 0, d.Lx, 0);
-            } else {
-                const int NL = generic_rows_nl<T>(d.Lx);
-                const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(C);
-                smem_attr((const void*)k_rows<T, -1>, sm);
-                k_rows<T, -1><<<dim3(cdiv(nrows, NL), nsys), NTH, sm, st>>>(pl.px, (const C*)pl.twx, sys, 2, 3, nrows, NL,
-                                                                             d.nx, 0, d.Lx, 0);
-            }
-        }, fourstep_prunable(d.Lx, d.nx, 0) ? 0 : 1);
-    }
+    launch_xrows<T>(d, sys, nsys, pl, 2, 3, 9LL * d.nz * d.ny, d.nx, st);
     ktimer_mark(tm, 1, f32, st, 1);
     // 3. forward y FFT: w2 -> w1 [9][nz][Ly][Lx]
     ktimer_mark(tm, 2, f32, st, 0);
@@ -1921,6 +1934,12 @@ cudaError_t fft3_inplace_setup(const Dims& d, const Plans& pl, double2* buf, int
         k_strided_raw<double, -1><<<dim3(cdiv(d.Lx, a.TX), d.Ly, ncomp), NTH, sm, st>>>(pl.pz, (const C*)pl.twz, a, buf, buf);
     }
     if (nl) *nl += 3;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fx_spectrum(const double2* ghat64, long long NO, int4* gx, int* ge, cudaStream_t st, long long* nl) {
+    k_fx_spectrum<<<grid_elems(NO), NTH, 0, st>>>(ghat64, NO, gx, ge);
+    if (nl) *nl += 1;
     return cudaGetLastError();
 }
 

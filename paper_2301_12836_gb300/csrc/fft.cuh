@@ -16,6 +16,7 @@
 // Forward is dir = -1 (numpy's convention); inverse is dir = +1 and unnormalised.
 #pragma once
 #include "dfloat.cuh"
+#include "fx.cuh"
 
 namespace lsm {
 
@@ -25,11 +26,17 @@ template <int S, typename C> __device__ __forceinline__ void bfly2(C* v) {
     v[0] = cadd(a, b); v[1] = csub(a, b);
 }
 
+// a + S i b, a - S i b
+template <int S, typename C> __device__ __forceinline__ C caddi(C a, C b) { return cadd(a, cmul_si<S>(b)); }
+template <int S, typename C> __device__ __forceinline__ C csubi(C a, C b) { return csub(a, cmul_si<S>(b)); }
+template <int S> __device__ __forceinline__ fxc caddi(fxc a, fxc b) { return fx_addi<S>(a, b); }
+template <int S> __device__ __forceinline__ fxc csubi(fxc a, fxc b) { return fx_subi<S>(a, b); }
+
 template <int S, typename C> __device__ __forceinline__ void bfly4(C* v) {
     C t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
-    C t2 = cadd(v[1], v[3]), t3 = cmul_si<S>(csub(v[1], v[3]));
+    C t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
     v[0] = cadd(t0, t2); v[2] = csub(t0, t2);
-    v[1] = cadd(t1, t3); v[3] = csub(t1, t3);
+    v[1] = caddi<S>(t1, t3); v[3] = csubi<S>(t1, t3);
 }
 
 // 4-point DFT whose inputs NZ..3 are zero (NZ = 1..4), computing only its first NO outputs
@@ -51,23 +58,23 @@ template <int S, int NZ, int NO, typename C> __device__ __forceinline__ void bfl
         }
         if constexpr (NZ == 4) {
             t2 = cadd(v[1], v[3]);
-            t3 = cmul_si<S>(csub(v[1], v[3]));
+            t3 = csub(v[1], v[3]);
         } else {
             t2 = v[1];
-            t3 = cmul_si<S>(v[1]);
+            t3 = v[1];
         }
         v[0] = cadd(t0, t2);
-        if constexpr (NO >= 2) v[1] = cadd(t1, t3);
+        if constexpr (NO >= 2) v[1] = caddi<S>(t1, t3);
         if constexpr (NO >= 3) v[2] = csub(t0, t2);
-        if constexpr (NO >= 4) v[3] = csub(t1, t3);
+        if constexpr (NO >= 4) v[3] = csubi<S>(t1, t3);
     }
 }
 
 // 4-point DFT of (v0, v1, 0, 0): the first radix-2 layer has nothing to add.
 template <int S, typename C> __device__ __forceinline__ void bfly4_half(C* v) {
-    const C a = v[0], b = v[1], bi = cmul_si<S>(v[1]);
+    const C a = v[0], b = v[1];
     v[0] = cadd(a, b); v[2] = csub(a, b);
-    v[1] = cadd(a, bi); v[3] = csub(a, bi);
+    v[1] = caddi<S>(a, b); v[3] = csubi<S>(a, b);
 }
 
 // HALF: inputs 4..7 are zero (zero-padded lines), so each 4-point half-DFT has two zero inputs.
@@ -121,9 +128,58 @@ template <int S, typename C> __device__ __forceinline__ void bfly5(C* v) {
     v[2] = cadd(m2, n2); v[3] = csub(m2, n2);
 }
 
-template <int S, int R, typename C>
+// Fixed-point forms of the butterflies with constants of their own (fx.cuh); bfly2, bfly4, bfly4p
+// and the 16- and 32-point DFTs only add and call cmul_const, so the templates serve both.
+template <int S, bool HALF = false> __device__ __forceinline__ void bfly8(fxc* v) {
+    const double r2 = 0.70710678118654752440;
+    fxc e[4] = {v[0], v[2], v[4], v[6]};
+    fxc o[4] = {v[1], v[3], v[5], v[7]};
+    if (HALF) {
+        bfly4_half<S>(e);
+        bfly4_half<S>(o);
+    } else {
+        bfly4<S>(e);
+        bfly4<S>(o);
+    }
+    const fxc o1 = cmul_const<S>(o[1], r2, r2), o3 = cmul_const<S>(o[3], -r2, r2);
+    v[0] = cadd(e[0], o[0]);     v[4] = csub(e[0], o[0]);
+    v[1] = cadd(e[1], o1);       v[5] = csub(e[1], o1);
+    v[2] = fx_addi<S>(e[2], o[2]); v[6] = fx_subi<S>(e[2], o[2]);
+    v[3] = cadd(e[3], o3);   v[7] = csub(e[3], o3);
+}
+__device__ __forceinline__ fxc fx_cscale(fxc a, double c) {
+    const long long k = fx_const(c < 0 ? -c : c);
+    const fxc r{fx_scale(a.x, k), fx_scale(a.y, k)};
+    return c < 0 ? fxc{fx_neg(r.x), fx_neg(r.y)} : r;
+}
+template <int S> __device__ __forceinline__ void bfly3(fxc* v) {
+    const fxc t = cadd(v[1], v[2]);
+    const fxc d = fx_cscale(csub(v[1], v[2]), 0.86602540378443864676);
+    // v0 - t / 2, the half rounded upwards
+    const fxc h{fx_r((fx_ll(t.x) + 1) >> 1), fx_r((fx_ll(t.y) + 1) >> 1)};
+    const fxc m = csub(v[0], h);
+    v[0] = cadd(v[0], t);
+    v[1] = fx_addi<S>(m, d);
+    v[2] = fx_subi<S>(m, d);
+}
+template <int S> __device__ __forceinline__ void bfly5(fxc* v) {
+    const double c1 = 0.30901699437494742410, c2 = -0.80901699437494742410;
+    const double s1 = 0.95105651629515357212, s2 = 0.58778525229247312917;
+    const fxc a14 = cadd(v[1], v[4]), b14 = csub(v[1], v[4]);
+    const fxc a23 = cadd(v[2], v[3]), b23 = csub(v[2], v[3]);
+    const fxc m1 = cadd(v[0], cadd(fx_cscale(a14, c1), fx_cscale(a23, c2)));
+    const fxc m2 = cadd(v[0], cadd(fx_cscale(a14, c2), fx_cscale(a23, c1)));
+    const fxc n1 = cadd(fx_cscale(b14, s1), fx_cscale(b23, s2));
+    const fxc n2 = csub(fx_cscale(b14, s2), fx_cscale(b23, s1));
+    v[0] = cadd(v[0], cadd(a14, a23));
+    v[1] = fx_addi<S>(m1, n1); v[4] = fx_subi<S>(m1, n1);
+    v[2] = fx_addi<S>(m2, n2); v[3] = fx_subi<S>(m2, n2);
+}
+
+// Tw: the twiddle table's entry type (C itself, or int4 for fixed point)
+template <int S, int R, typename C, typename Tw>
 __device__ __forceinline__ void fft_stage_r(const C* __restrict__ src, C* __restrict__ dst, int L, int Ns,
-                                            int NL, int LD, const C* __restrict__ tw, int tid, int nth) {
+                                            int NL, int LD, const Tw* __restrict__ tw, int tid, int nth) {
     const int nb = L / R;
     const int total = nb * NL;
     const int tstep = L / (Ns * R);
@@ -136,11 +192,7 @@ __device__ __forceinline__ void fft_stage_r(const C* __restrict__ src, C* __rest
         for (int r = 0; r < R; ++r) v[r] = src[(j + r * nb) * LD + l];
         if (k) {
 #pragma unroll
-            for (int r = 1; r < R; ++r) {
-                C w = __ldg(&tw[r * k * tstep]);
-                if (S > 0) w.y = -w.y;
-                v[r] = cmul(v[r], w);
-            }
+            for (int r = 1; r < R; ++r) v[r] = tw_mul<S>(v[r], tw, r * k * tstep);
         }
         if (R == 2) bfly2<S>(v);
         else if (R == 3) bfly3<S>(v);
@@ -156,8 +208,8 @@ __device__ __forceinline__ void fft_stage_r(const C* __restrict__ src, C* __rest
 // Transform NL lines of length p.L held in buffer a (layout s[e*LD + l]); b is scratch of the
 // same size.  Returns the buffer holding the result.  The caller synchronises the block before
 // the call; the result is visible to all threads on return.  tw = exp(-2 pi i k / L), k < L.
-template <int S, typename C>
-__device__ C* fft_smem(C* a, C* b, const FftPlan& p, int NL, int LD, const C* __restrict__ tw, int tid, int nth) {
+template <int S, typename C, typename Tw>
+__device__ C* fft_smem(C* a, C* b, const FftPlan& p, int NL, int LD, const Tw* __restrict__ tw, int tid, int nth) {
     int Ns = 1;
     for (int s = 0; s < p.nst; ++s) {
         const int R = p.radix[s];

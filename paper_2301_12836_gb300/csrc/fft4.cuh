@@ -9,6 +9,7 @@
 // threads: thread tid works on line tid % NL.  Line l, element e sits at s[e * LD + l].
 #pragma once
 #include "fft.cuh"
+#include <type_traits>
 
 namespace lsm {
 
@@ -201,8 +202,8 @@ template <int A, int B> struct FourStep {
 // Zero padding and cropping are pruned at compile time: elements e >= NZ * B of a line are known
 // to be zero (each step-1 DFT has at most NZ nonzero inputs), and only outputs k < NO * A are
 // wanted (each step-2 DFT produces its first NO outputs; the others are left unwritten).
-template <int A, int B, int S, int NZ = A, int NO = B, typename C>
-__device__ __forceinline__ void fft4_smem(C* s, int NL, int LD, const C* __restrict__ tw, int tid) {
+template <int A, int B, int S, int NZ = A, int NO = B, typename C, typename Tw>
+__device__ __forceinline__ void fft4_smem(C* s, int NL, int LD, const Tw* __restrict__ tw, int tid) {
     typedef FourStep<A, B> F;
     const int l = tid % NL;
     const int q = tid / NL;
@@ -213,14 +214,7 @@ __device__ __forceinline__ void fft4_smem(C* s, int NL, int LD, const C* __restr
 #pragma unroll
         for (int a = 0; a < A; ++a) v[i][a] = a < NZ ? s[(t + B * a) * LD + l] : czero<C>();
         dft_reg_p<A, S, NZ, A>(v[i]);
-        if (t) {
-#pragma unroll
-            for (int k1 = 1; k1 < A; ++k1) {
-                C w = __ldg(&tw[t * k1]);
-                if (S > 0) w.y = -w.y;
-                v[i][k1] = cmul(v[i][k1], w);
-            }
-        }
+        tw_row<S, A * B, A>(v[i], tw, t);
     }
     __syncthreads();
 #pragma unroll
@@ -265,39 +259,25 @@ __host__ __device__ constexpr int fft4_ystride(int NL) {
     return A * NL + fft4_pad<A, (int)(128 / sizeof(C))>(NL);
 }
 
-// Four-step FFT with caller-supplied input and output.  ld(l, e) returns element e of line l
-// (IN_SMEM: it reads the buffer s itself, so a barrier separates those reads from the first
-// write into s); st(l, k, v) receives output k of line l (OUT_SMEM: it writes s, so a barrier
-// separates the last reads of s from those writes).  Called by exactly NL * TPL threads.  The
-// intermediate occupies B * fft4_ystride<A, C>(NL) elements of s.  As in fft4_smem, inputs
-// e >= NZ * B are known to be zero (ld is not called for them) and only outputs k < NO * A are
-// produced (st is not called for the others).
-template <int A, int B, int S, bool IN_SMEM, bool OUT_SMEM, int NL, int NZ = A, int NO = B, typename C, class Ld,
-          class St>
-__device__ __forceinline__ void fft4_io(C* s, const C* __restrict__ tw, int tid, Ld ld, St st) {
+// fft4_io's transform of step-1 inputs already in registers: v[i][a] = element t + B a of line
+// tid % NL, t = tid / NL + TPL i.
+// Fixed point with an output of its own form (ODD: st takes a fourth argument whose call is a
+// constant): a line whose outputs need the careful conversion (odd) stores in a second loop.
+struct fft4_plain {};
+template <bool V> struct fft4_flag {
+    __device__ __forceinline__ constexpr bool operator()() const { return V; }
+};
+template <int A, int B, int S, bool IN_SMEM, bool OUT_SMEM, int NL, int NZ = A, int NO = B, typename C, typename Tw, class St, class Odd = fft4_plain>
+__device__ __forceinline__ void fft4_run(C (&v)[FourStep<A, B>::I1][A], C* s, const Tw* __restrict__ tw, int tid, St st, Odd odd = Odd()) {
     typedef FourStep<A, B> F;
     const int l = tid % NL;
     const int q = tid / NL;
     constexpr int YS = fft4_ystride<A, C>(NL);
-    C v[F::I1][A];
-#pragma unroll
-    for (int i = 0; i < F::I1; ++i) {
-        const int t = q + F::TPL * i;
-#pragma unroll
-        for (int a = 0; a < A; ++a) v[i][a] = a < NZ ? ld(l, t + B * a) : czero<C>();
-    }
 #pragma unroll
     for (int i = 0; i < F::I1; ++i) {
         const int t = q + F::TPL * i;
         dft_reg_p<A, S, NZ, A>(v[i]);
-        if (t) {
-#pragma unroll
-            for (int k1 = 1; k1 < A; ++k1) {
-                C w = __ldg(&tw[t * k1]);
-                if (S > 0) w.y = -w.y;
-                v[i][k1] = cmul(v[i][k1], w);
-            }
-        }
+        tw_row<S, A * B, A>(v[i], tw, t);
     }
     if (IN_SMEM) __syncthreads();
 #pragma unroll
@@ -319,10 +299,41 @@ __device__ __forceinline__ void fft4_io(C* s, const C* __restrict__ tw, int tid,
 #pragma unroll
     for (int i = 0; i < F::I2; ++i) {
         const int k1 = q + F::TPL * i;
+        if constexpr (std::is_same<Odd, fft4_plain>::value) {
 #pragma unroll
-        for (int k2 = 0; k2 < NO; ++k2) st(l, k1 + A * k2, w2[i][k2]);
+            for (int k2 = 0; k2 < NO; ++k2) st(l, k1 + A * k2, w2[i][k2]);
+        } else if (!odd) {
+#pragma unroll
+            for (int k2 = 0; k2 < NO; ++k2) st(l, k1 + A * k2, w2[i][k2], fft4_flag<false>());
+        } else {
+#pragma unroll
+            for (int k2 = 0; k2 < NO; ++k2) st(l, k1 + A * k2, w2[i][k2], fft4_flag<true>());
+        }
     }
     if (OUT_SMEM) __syncthreads();
+}
+
+// Four-step FFT with caller-supplied input and output.  ld(l, e) returns element e of line l
+// (IN_SMEM: it reads the buffer s itself, so a barrier separates those reads from the first
+// write into s); st(l, k, v) receives output k of line l (OUT_SMEM: it writes s, so a barrier
+// separates the last reads of s from those writes).  Called by exactly NL * TPL threads.  The
+// intermediate occupies B * fft4_ystride<A, C>(NL) elements of s.  As in fft4_smem, inputs
+// e >= NZ * B are known to be zero (ld is not called for them) and only outputs k < NO * A are
+// produced (st is not called for the others).
+template <int A, int B, int S, bool IN_SMEM, bool OUT_SMEM, int NL, int NZ = A, int NO = B, typename C, typename Tw, class Ld,
+          class St>
+__device__ __forceinline__ void fft4_io(C* s, const Tw* __restrict__ tw, int tid, Ld ld, St st) {
+    typedef FourStep<A, B> F;
+    const int l = tid % NL;
+    const int q = tid / NL;
+    C v[F::I1][A];
+#pragma unroll
+    for (int i = 0; i < F::I1; ++i) {
+        const int t = q + F::TPL * i;
+#pragma unroll
+        for (int a = 0; a < A; ++a) v[i][a] = a < NZ ? ld(l, t + B * a) : czero<C>();
+    }
+    fft4_run<A, B, S, IN_SMEM, OUT_SMEM, NL, NZ, NO>(v, s, tw, tid, st);
 }
 
 }  // namespace lsm

@@ -16,6 +16,8 @@ struct ApplySys {
                          // then, in the sampled-H form, H_iJ at plane 6 + 6 i + J
     C* w1;               // workspace (see apply_ws_elems)
     C* w2;               // workspace
+    const int4* gx = nullptr;  // FP64 only: fixed-point copy of the six G spectra (apply_fx.cuh) ...
+    const int* ge = nullptr;   // ... and its exponent per point
     T omega2;            // w^2
     const int* run;      // system runs when run == nullptr or *run != 0
     unsigned long long* count;  // incremented once per executed system apply (may be nullptr)
@@ -54,6 +56,8 @@ struct Plans {
     const void* twx;     // twiddle tables of T: exp(-2 pi i k / L)
     const void* twy;
     const void* twz;
+    // FP64 plans: the same tables as two-word fixed-point numbers (fx.cuh)
+    const int4 *fxx = nullptr, *fxy = nullptr, *fxz = nullptr;
 };
 
 // workspace elements (complex) needed by one system's apply / adjoint in w1 and w2 (kernel as in Medium)
@@ -107,6 +111,9 @@ cudaError_t launch_time_traces(int nf, double df, int ntr, const double2* U, int
 // Receiver gather for the seismogram chain: out[r * 3 + c] = u[c * N + node[r]], r < nrec (FP64).
 cudaError_t launch_gather_receivers(const double2* u, long long N, const long long* node, int nrec, double2* out,
                                     cudaStream_t st);
+
+// Fixed-point copy of six FP64 octant spectra for the z pass: gx [6][NO], ge [NO] (apply_fx.cuh).
+cudaError_t launch_fx_spectrum(const double2* ghat64, long long NO, int4* gx, int* ge, cudaStream_t st, long long* nlaunch);
 
 // Precision converters.  d2df: n reals to double-float pairs; df2d_inplace: n double-float pairs
 // to doubles in the same memory (8 bytes each).

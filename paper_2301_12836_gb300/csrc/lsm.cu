@@ -6,6 +6,7 @@
 // runs in the kernels of apply.cu, green.cu and solver.cu.
 #include "lsm.h"
 #include "kernels.h"
+#include "fx.cuh"
 #include "solver.cuh"
 
 #include <cmath>
@@ -84,6 +85,7 @@ struct Store {
     float* drho32 = nullptr;
     Plans pl64, pl32, pldf;
     double2* tw64 = nullptr;
+    int4* twfx = nullptr;            // tw64 as two-word fixed-point numbers
     float2* tw32 = nullptr;
     // double-float copies for the mixed refinement residual (LSM_RESIDUAL_DFLOAT)
     bool pair = false;
@@ -115,6 +117,8 @@ struct lsm_ctx {
     double omega = 0;
     lsm_opts o;
     double2* ghat64 = nullptr;
+    int4* gx = nullptr;       // fixed-point copy of the G spectra for the FP64 z pass, and ...
+    int* ge = nullptr;        // ... its exponent per point
     float2* ghat32 = nullptr;
     dfcplx* ghatdf = nullptr;
     long long nl = 0;
@@ -154,14 +158,34 @@ bool factor_plan(int L, FftPlan& p) {
     return m == 1;
 }
 
-// exp(-2 pi i k / L), k < L, evaluated in long double and rounded once
-void twiddle_table(int L, std::vector<double2>& t64, std::vector<float2>& t32) {
+// v (|v| <= 1) as the two-word fixed-point number v1 2^-w + v0 2^-2w, both words within
+// +-(2^31 - 1) so that either sign can be negated
+void fx_words(long double v, int w, int* v1, int* v0) {
+    const long double lim = 2147483647.0L, f = (long double)(1LL << w);
+    long double a = nearbyintl(v * f);
+    a = a > lim ? lim : (a < -lim ? -lim : a);
+    long double b = nearbyintl((v * f - a) * f);
+    b = b > lim ? lim : (b < -lim ? -lim : b);
+    *v1 = (int)a;
+    *v0 = (int)b;
+}
+
+// exp(-2 pi i k / L), k < L, evaluated in long double and rounded once (the fixed-point table with
+// the two-step transforms' change of unit, fx.cuh)
+void twiddle_table(int L, std::vector<double2>& t64, std::vector<float2>& t32, std::vector<int4>& tfx) {
     const long double pi = 3.141592653589793238462643383279502884L;
     for (int k = 0; k < L; ++k) {
         const long double a = -2.0L * pi * (long double)k / (long double)L;
         const long double c = cosl(a), s = sinl(a);
         t64.push_back(make_double2((double)c, (double)s));
         t32.push_back(make_float2((float)c, (float)s));
+        // two-step plans: scaled to below 1/2, split at the words (fx_cmul32); generic plans: fx_cmul
+        const int K = fx_prescale(L);
+        const long double f = 1.0L / (1 << K);
+        int4 w;
+        fx_words(c * f, K ? 32 : 31, &w.x, &w.y);
+        fx_words(s * f, K ? 32 : 31, &w.z, &w.w);
+        tfx.push_back(w);
     }
 }
 
@@ -175,7 +199,7 @@ void store_release(Store* s) {
     if (!s) return;
     if (--s->refs > 0) return;
     cudaFree(s->dC64); cudaFree(s->drho64); cudaFree(s->dC32); cudaFree(s->drho32);
-    cudaFree(s->tw64); cudaFree(s->tw32);
+    cudaFree(s->tw64); cudaFree(s->tw32); cudaFree(s->twfx);
     cudaFree(s->dCdf); cudaFree(s->drhodf); cudaFree(s->twdf); cudaFree(s->udf); cudaFree(s->adf);
     cudaFree(s->w1_64); cudaFree(s->w2_64); cudaFree(s->w1_32); cudaFree(s->w2_32);
     cudaFree(s->a64); cudaFree(s->a32); cudaFree(s->flag); cudaFree(s->counts); cudaFree(s->grad_scratch);
@@ -295,6 +319,12 @@ static lsm_status build_spectrum(lsm_t h) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
     cudaFree(scratch);
     if (e != cudaSuccess) return cuda_fail(h, e, "green spectrum setup");
+    if (s->kernel == LSM_KERNEL_DIFF) {
+        CK(h, cudaMalloc(&h->gx, 6 * NO * sizeof(int4)));
+        CK(h, cudaMalloc(&h->ge, NO * sizeof(int)));
+        CK(h, launch_fx_spectrum(h->ghat64, NO, h->gx, h->ge, s->st, &h->nl));
+        CK(h, cudaStreamSynchronize(s->st));
+    }
     if (s->precision == LSM_MIXED) {
         CK(h, cudaMalloc(&h->ghat32, planes * NO * sizeof(float2)));
         CK(h, launch_d2f((const double*)h->ghat64, (float*)h->ghat32, 2 * planes * NO, s->st, &h->nl));
@@ -362,9 +392,13 @@ extern "C" lsm_status lsm_create(lsm_t* out, const int n[3], double dx, double l
         s->pl32.px = s->pl64.px; s->pl32.py = s->pl64.py; s->pl32.pz = s->pl64.pz;
         std::vector<double2> t64;
         std::vector<float2> t32;
-        twiddle_table(d.Lx, t64, t32);
-        twiddle_table(d.Ly, t64, t32);
-        twiddle_table(d.Lz, t64, t32);
+        std::vector<int4> tfx;
+        twiddle_table(d.Lx, t64, t32, tfx);
+        twiddle_table(d.Ly, t64, t32, tfx);
+        twiddle_table(d.Lz, t64, t32, tfx);
+        CKB(cudaMalloc(&s->twfx, tfx.size() * sizeof(int4)));
+        CKB(cudaMemcpy(s->twfx, tfx.data(), tfx.size() * sizeof(int4), cudaMemcpyHostToDevice));
+        s->pl64.fxx = s->twfx; s->pl64.fxy = s->twfx + d.Lx; s->pl64.fxz = s->twfx + d.Lx + d.Ly;
         CKB(cudaMalloc(&s->tw64, t64.size() * sizeof(double2)));
         CKB(cudaMalloc(&s->tw32, t32.size() * sizeof(float2)));
         CKB(cudaMemcpy(s->tw64, t64.data(), t64.size() * sizeof(double2), cudaMemcpyHostToDevice));
@@ -440,6 +474,8 @@ extern "C" lsm_status lsm_create_shared(lsm_t* out, lsm_t base, double omega) {
 extern "C" void lsm_destroy(lsm_t h) {
     if (!h) return;
     cudaFree(h->ghat64);
+    cudaFree(h->gx);
+    cudaFree(h->ge);
     cudaFree(h->ghat32);
     cudaFree(h->ghatdf);
     store_release(h->s);
@@ -498,6 +534,8 @@ static lsm_status apply_one(lsm_t h, const void* u, void* Au, bool adjoint) {
     a.u = (const C*)u;
     a.out = (C*)Au;
     a.ghat = f32 ? (const C*)h->ghat32 : (const C*)h->ghat64;
+    a.gx = h->gx;
+    a.ge = h->ge;
     a.w1 = f32 ? (C*)s->w1_32 : (C*)s->w1_64;
     a.w2 = f32 ? (C*)s->w2_32 : (C*)s->w2_64;
     a.omega2 = (T)(h->omega * h->omega);
@@ -854,6 +892,8 @@ static lsm_status solve_batched(int nsys, const lsm_t* hs_in, const void* const*
             ApplySys<double> a;
             a.count = s->counts;
             a.ghat = hs[i]->ghat64;
+            a.gx = hs[i]->gx;
+            a.ge = hs[i]->ge;
             a.w1 = (double2*)w.w1[i];
             a.w2 = (double2*)w.w2[i];
             a.omega2 = hs[i]->omega * hs[i]->omega;
@@ -922,6 +962,8 @@ static lsm_status solve_batched(int nsys, const lsm_t* hs_in, const void* const*
             ApplySys<double> d;
             d.count = s->counts;
             d.ghat = hs[i]->ghat64;
+            d.gx = hs[i]->gx;
+            d.ge = hs[i]->ge;
             d.w1 = w.w1d[i];
             d.w2 = w.w2d[i];
             d.omega2 = hs[i]->omega * hs[i]->omega;
@@ -1070,6 +1112,8 @@ extern "C" lsm_status lsm_gradient(lsm_t h, const void* u, const void* lam, doub
     a.u = (const double2*)lam;
     a.out = nullptr;
     a.ghat = h->ghat64;
+    a.gx = h->gx;
+    a.ge = h->ge;
     a.w1 = s->w1_64;
     a.w2 = s->w2_64;
     a.omega2 = h->omega * h->omega;
@@ -1152,6 +1196,8 @@ static lsm_status tune_one(lsm_t h, int nsys, int reps, const void* u, void* out
         a[i].u = (const C*)u;
         a[i].out = (C*)((char*)out + (size_t)i * 3 * s->d.N * sizeof(C));
         a[i].ghat = f32 ? (const C*)h->ghat32 : (const C*)h->ghat64;
+        a[i].gx = h->gx;
+        a[i].ge = h->ge;
         const bool fp64_of_mixed = !f32 && s->precision == LSM_MIXED;
         a[i].w1 = fp64_of_mixed ? (C*)w.w1d[i] : (C*)w.w1[i];
         a[i].w2 = fp64_of_mixed ? (C*)w.w2d[i] : (C*)w.w2[i];
@@ -1389,6 +1435,8 @@ extern "C" lsm_status lsm_apply_static(lsm_t h, const void* u, void* Au) {
     a.u = (const double2*)u;
     a.out = (double2*)Au;
     a.ghat = h->ghat64;
+    a.gx = h->gx;
+    a.ge = h->ge;
     a.w1 = w1;
     a.w2 = w2;
     a.omega2 = h->omega * h->omega;
