@@ -342,6 +342,7 @@ __global__ void __launch_bounds__(NTH) k_strided_raw(FftPlan p, const typename c
 
 }  // namespace lsm
 #include "apply_fx.cuh"
+#include "apply_fxg.cuh"
 namespace lsm {
 
 // four-step strided pass: step 1 loads straight from global memory, the last step stores straight
@@ -1370,26 +1371,68 @@ static void strided_cfg(int L, int ncomp, int& TX, int& threads, size_t& sm, int
     }
 }
 
-// forward x FFT of nrows rows of in_count elements, zero-padded to Lx: src_sel -> dst_sel [nrows][Lx]
-template <typename T>
+constexpr size_t FX_STATIC_SM = 256;   // at least the fixed-point kernels' static shared memory
+
+// Fixed-point tables of axis a, and the one the two-step plan of length L uses
+static inline FxTables fx_tables(const Plans& pl, int a) { return FxTables{pl.fx2[a], pl.fx3[a]}; }
+static inline const int4* fx_twostep(const Plans& pl, int a, int L) { return fx_prescale(L) == 2 ? pl.fx2[a] : pl.fx3[a]; }
+
+// Width (lines) of a generic fixed-point tile: the widest of 8, 4, 2 (at most `most`) whose two buffers
+// fit `cap` bytes; half of it for schedule variant 2.  The z pass takes 4 columns up to L = 128 and 2
+// beyond, where the smaller tile lets four blocks share an SM: 96^3 0.76 -> 0.65 ms, 100^3 0.91 -> 0.82
+// ms; at L = 100 (60 x 45 x 50) 4 columns are faster, 0.107 against 0.135 ms.
+static inline int fxg_width(int L, int per, int most, size_t cap, int v) {
+    int w = most;
+    while (w > 2 && 2 * (size_t)L * (per * w + 1) * sizeof(fxc) > cap) w /= 2;
+    if (v == 2 && w > 2) w /= 2;
+    return w;
+}
+template <typename Fn> static void with_width(int w, Fn&& fn) {
+    if (w == 8) fn(std::integral_constant<int, 8>());
+    else if (w == 4) fn(std::integral_constant<int, 4>());
+    else fn(std::integral_constant<int, 2>());
+}
+
+// FP64 rows through the generic fixed-point engine; OUT as in kg_rows_fx
+template <int DIR, bool OUT>
+static void launch_rows_fxg(const Dims& d, const ApplySys<double>* sys, int nsys, const Plans& pl, int src_sel, int dst_sel,
+                            long long nrows, int in_count, int in_off, int out_count, int out_off, cudaStream_t st, int v) {
+    with_width(fxg_width(d.Lx, 1, 8, SMEM_CAP, v), [&](auto w) {
+        constexpr int NL = decltype(w)::value;
+        const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(fxc);
+        const int m = fxg_groups(pl.px, 64 / NL, NL < 4 ? 48 : 192 / NL);
+        smem_attr((const void*)kg_rows_fx<DIR, NL, OUT>, sm, FX_STATIC_SM);
+        kg_rows_fx<DIR, NL, OUT><<<dim3(cdiv(nrows, NL), nsys), NL * m, sm, st>>>(
+            pl.px, fx_tables(pl, 0), sys, src_sel, dst_sel, nrows, in_count, in_off, out_count, out_off);
+    });
+}
+
+// x FFT of nrows contiguous rows: in_count elements at in_off of each line (forward: the rest zero),
+// outputs out_off .. out_off + out_count - 1: src_sel -> dst_sel
+template <typename T, int DIR>
 static void launch_xrows(const Dims& d, const ApplySys<T>* sys, int nsys, const Plans& pl, int src_sel, int dst_sel,
-                         long long nrows, int in_count, cudaStream_t st, int v = 0) {
+                         long long nrows, int in_count, int in_off, int out_count, int out_off, cudaStream_t st, int v = 0) {
     typedef typename cplx_of<T>::type C;
-    if (!fourstep_prunable(d.Lx, in_count, 0)) v = 1;
+    if (!fourstep_prunable(d.Lx, DIR < 0 ? in_off + in_count : 0, DIR > 0 ? out_off + out_count : 0)) v = 1;
     with_engine<std::is_same<T, dfloat>::value>(d.Lx, [&](auto eng) {
         using F = decltype(eng);
-        if constexpr (F::INPLACE && std::is_same<T, double>::value) {
-            constexpr int A = F::A_, B = F::B_, LPB = 128 / F::TPL;
-            const size_t sm = (size_t)LPB * B * (A + 1) * sizeof(fxc);
-            smem_attr((const void*)k4_rows_fx<A, B, LPB>, sm);
-            k4_rows_fx<A, B, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * F::TPL, sm, st>>>(
-                pl.fxx, sys, src_sel, dst_sel, nrows, in_count, fx_bits(A * B, in_count, A / 2 + 1, B));
+        if constexpr (std::is_same<T, double>::value) {
+            if constexpr (F::INPLACE) {
+                constexpr int A = F::A_, B = F::B_, LPB = 128 / F::TPL;
+                const size_t sm = (size_t)LPB * B * (A + 1) * sizeof(fxc);
+                smem_attr((const void*)k4_rows_fx<DIR, A, B, LPB>, sm, FX_STATIC_SM);
+                k4_rows_fx<DIR, A, B, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * F::TPL, sm, st>>>(
+                    fx_twostep(pl, 0, A * B), sys, src_sel, dst_sel, nrows, in_count, in_off, out_count, out_off,
+                    fx_bits(A * B, in_count, DIR < 0 ? A / 2 + 1 : A, B));
+            } else {
+                launch_rows_fxg<DIR, false>(d, sys, nsys, pl, src_sel, dst_sel, nrows, in_count, in_off, out_count, out_off, st, v);
+            }
         } else if constexpr (F::INPLACE && F::A_ == F::B_) {
             constexpr int A = F::A_, LPB = sizeof(T) == 4 ? 16 : 8;
             k4_rows_w<T, A, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * A, 0, st>>>((const C*)pl.twx, sys, src_sel, dst_sel,
                                                                                    nrows, in_count);
         } else if constexpr (F::INPLACE) {
-            constexpr int A = F::A_, B = F::B_, NL = sizeof(T) == 4 ? 8 : 12;
+            constexpr int A = F::A_, B = F::B_, NL = 8 + (sizeof(T) == 4 ? 0 : 4);
             const size_t sm = (size_t)A * B * (NL + 1) * sizeof(C);
             smem_attr((const void*)k4_rows<T, -1, A, B, NL>, sm);
             k4_rows<T, -1, A, B, NL><<<dim3(cdiv(nrows, NL), nsys), NL * F::TPL, sm, st>>>(
@@ -1397,9 +1440,9 @@ static void launch_xrows(const Dims& d, const ApplySys<T>* sys, int nsys, const 
         } else {
             const int NL = generic_rows_nl<T>(d.Lx, v == 2);
             const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(C);
-            smem_attr((const void*)k_rows<T, -1>, sm);
-            k_rows<T, -1><<<dim3(cdiv(nrows, NL), nsys), NTH, sm, st>>>(pl.px, (const C*)pl.twx, sys, src_sel, dst_sel, nrows,
-                                                                         NL, in_count, 0, d.Lx, 0);
+            smem_attr((const void*)k_rows<T, DIR>, sm);
+            k_rows<T, DIR><<<dim3(cdiv(nrows, NL), nsys), NTH, sm, st>>>(pl.px, (const C*)pl.twx, sys, src_sel, dst_sel, nrows,
+                                                                         NL, in_count, in_off, out_count, out_off);
         }
     }, v);
 }
@@ -1407,7 +1450,7 @@ static void launch_xrows(const Dims& d, const ApplySys<T>* sys, int nsys, const 
 // forward x FFT of the contrast source rows: w2 [3][ez][ey][ex] -> w1 [3][ez][ey][Lx]
 template <typename T>
 static void launch_xfwd(const Dims& d, const ApplySys<T>* sys, int nsys, const Plans& pl, cudaStream_t st, int v = 0) {
-    launch_xrows<T>(d, sys, nsys, pl, 3, 2, 3LL * d.ez * d.ey, d.ex, st, v);
+    launch_xrows<T, -1>(d, sys, nsys, pl, 3, 2, 3LL * d.ez * d.ey, d.ex, 0, d.Lx, 0, st, v);
 }
 
 // xoff: padded-grid index of model node 0 (1 when the convolved source lives on the extended nodes)
@@ -1420,12 +1463,17 @@ static void launch_fftx_out(const Dims& d, const ApplySys<T>* sys, int nsys, con
     typedef typename cplx_of<T>::type C;
     with_engine<std::is_same<T, dfloat>::value>(d.Lx, [&](auto eng) {
         using F = decltype(eng);
-        if constexpr (F::INPLACE && std::is_same<T, double>::value) {
-            constexpr int A = F::A_, B = F::B_, LPB = 128 / F::TPL;
-            const size_t sm = (size_t)LPB * B * (A + 1) * sizeof(fxc);
-            smem_attr((const void*)k4_xout_fx<A, B, LPB>, sm);
-            k4_xout_fx<A, B, LPB><<<dim3(cdiv(3LL * d.nz * d.ny, LPB), nsys), LPB * F::TPL, sm, st>>>(
-                d, sys, pl.fxx, xoff, fx_bits(A * B, A * B, A, B));
+        if constexpr (std::is_same<T, double>::value) {
+            const long long nrows = 3LL * d.nz * d.ny;
+            if constexpr (F::INPLACE) {
+                constexpr int A = F::A_, B = F::B_, LPB = 128 / F::TPL;
+                const size_t sm = (size_t)LPB * B * (A + 1) * sizeof(fxc);
+                smem_attr((const void*)k4_xout_fx<A, B, LPB>, sm, FX_STATIC_SM);
+                k4_xout_fx<A, B, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * F::TPL, sm, st>>>(
+                    d, sys, fx_twostep(pl, 0, A * B), xoff, fx_bits(A * B, A * B, A, B));
+            } else {
+                launch_rows_fxg<1, true>(d, sys, nsys, pl, 3, 1, nrows, d.Lx, 0, d.nx, xoff, st, v);
+            }
         } else if constexpr (F::INPLACE && F::A_ == F::B_) {
             constexpr int A = F::A_, LPB = sizeof(T) == 4 ? 16 : 8;
             const long long nrows = 3LL * d.nz * d.ny;
@@ -1463,27 +1511,41 @@ static void launch_fftx_out(const Dims& d, const ApplySys<T>* sys, int nsys, con
 // Plain FFT of lines of length L along a strided axis: a.ncomp components per system, lines along
 // x (a.nlines of them), `outer` line groups (blockIdx.y) per component.
 template <typename T, int DIR>
-static void launch_strided(int L, const FftPlan& p, const void* tw, const int4* fxtw, StridedArgs a, int outer,
+static void launch_strided(int L, const FftPlan& p, const void* tw, const Plans& pl, int axis, StridedArgs a, int outer,
                            const ApplySys<T>* sys, int nsys, cudaStream_t st, int v = 0) {
     typedef typename cplx_of<T>::type C;
     if (!fourstep_prunable(L, DIR < 0 ? a.in_off + a.in_count : 0, DIR > 0 ? a.out_off + a.out_count : 0)) v = 1;
     with_engine<std::is_same<T, dfloat>::value>(L, [&](auto eng) {
         using F = decltype(eng);
-        int th;
-        size_t sm;
-        strided_cfg<T, F>(L, 1, a.TX, th, sm, v == 2);
-        if constexpr (F::INPLACE && std::is_same<T, double>::value) {
-            constexpr int A = F::A_, B = F::B_, TXC = 8;
-            smem_attr((const void*)k4_strided_fx<DIR, A, B, TXC>, sm);
-            k4_strided_fx<DIR, A, B, TXC><<<dim3(cdiv(a.nlines, TXC), outer, a.ncomp * nsys), th, sm, st>>>(
-                fxtw, a, sys, fx_bits(L, a.in_count, DIR < 0 ? A / 2 + 1 : A, B));
-        } else if constexpr (F::INPLACE) {
-            constexpr int A = F::A_, B = F::B_, TXC = sizeof(T) == 4 ? 16 : 8;
-            smem_attr((const void*)k4_strided<T, DIR, A, B, TXC>, sm);
-            k4_strided<T, DIR, A, B, TXC><<<dim3(cdiv(a.nlines, a.TX), outer, a.ncomp * nsys), th, sm, st>>>((const C*)tw, a, sys);
+        if constexpr (std::is_same<T, double>::value) {
+            if constexpr (F::INPLACE) {
+                constexpr int A = F::A_, B = F::B_, TXC = 8;
+                const size_t sm = (size_t)B * fft4_ystride<A, fxc>(TXC) * sizeof(fxc);
+                smem_attr((const void*)k4_strided_fx<DIR, A, B, TXC>, sm, FX_STATIC_SM);
+                k4_strided_fx<DIR, A, B, TXC><<<dim3(cdiv(a.nlines, TXC), outer, a.ncomp * nsys), TXC * F::TPL, sm, st>>>(
+                    fx_twostep(pl, axis, L), a, sys, fx_bits(L, a.in_count, DIR < 0 ? A / 2 + 1 : A, B));
+            } else {
+                with_width(fxg_width(L, 1, 8, SMEM_CAP, v), [&](auto w) {
+                    constexpr int NL = decltype(w)::value;
+                    const size_t sm = 2 * (size_t)L * NL * sizeof(fxc);
+                    const int m = fxg_groups(p, 64 / NL, NL < 4 ? 48 : 192 / NL);
+                    smem_attr((const void*)kg_strided_fx<DIR, NL>, sm, FX_STATIC_SM);
+                    kg_strided_fx<DIR, NL><<<dim3(cdiv(a.nlines, NL), outer, a.ncomp * nsys), NL * m, sm, st>>>(
+                        p, fx_tables(pl, axis), a, sys);
+                });
+            }
         } else {
-            smem_attr((const void*)k_strided<T, DIR, F>, sm);
-            k_strided<T, DIR, F><<<dim3(cdiv(a.nlines, a.TX), outer, a.ncomp * nsys), th, sm, st>>>(p, (const C*)tw, a, sys);
+            int th;
+            size_t sm;
+            strided_cfg<T, F>(L, 1, a.TX, th, sm, v == 2);
+            if constexpr (F::INPLACE) {
+                constexpr int A = F::A_, B = F::B_, TXC = sizeof(T) == 4 ? 16 : 8;
+                smem_attr((const void*)k4_strided<T, DIR, A, B, TXC>, sm);
+                k4_strided<T, DIR, A, B, TXC><<<dim3(cdiv(a.nlines, a.TX), outer, a.ncomp * nsys), th, sm, st>>>((const C*)tw, a, sys);
+            } else {
+                smem_attr((const void*)k_strided<T, DIR, F>, sm);
+                k_strided<T, DIR, F><<<dim3(cdiv(a.nlines, a.TX), outer, a.ncomp * nsys), th, sm, st>>>(p, (const C*)tw, a, sys);
+            }
         }
     }, v);
 }
@@ -1499,7 +1561,7 @@ static void launch_ypass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
     a.src_es = d.Lx; a.src_os1 = (long long)in_count * d.Lx; a.src_os2 = (long long)planes * in_count * d.Lx;
     a.dst_es = d.Lx; a.dst_os1 = (long long)out_count * d.Lx; a.dst_os2 = (long long)planes * out_count * d.Lx;
     a.ncomp = ncomp; a.src_sel = src_sel; a.dst_sel = dst_sel;
-    launch_strided<T, DIR>(d.Ly, pl.py, pl.twy, pl.fxy, a, planes, sys, nsys, st, v);
+    launch_strided<T, DIR>(d.Ly, pl.py, pl.twy, pl, 1, a, planes, sys, nsys, st, v);
 }
 
 // plain z pass: src [ncomp][in_count][Ly][Lx] (sel) -> dst [ncomp][out_count][Ly][Lx] (sel)
@@ -1513,7 +1575,7 @@ static void launch_zplain(const Dims& d, const ApplySys<T>* sys, int nsys, const
     a.src_es = plane; a.src_os1 = d.Lx; a.src_os2 = (long long)in_count * plane;
     a.dst_es = plane; a.dst_os1 = d.Lx; a.dst_os2 = (long long)out_count * plane;
     a.ncomp = ncomp; a.src_sel = src_sel; a.dst_sel = dst_sel;
-    launch_strided<T, DIR>(d.Lz, pl.pz, pl.twz, pl.fxz, a, d.Ly, sys, nsys, st);
+    launch_strided<T, DIR>(d.Lz, pl.pz, pl.twz, pl, 2, a, d.Ly, sys, nsys, st);
 }
 
 // schedule variant v: 0 default (register-resident kernel for FP32 and L = A * A), 1 / 2 generic
@@ -1525,6 +1587,26 @@ static void launch_zpass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
     typedef typename cplx_of<T>::type C;
     with_engine<std::is_same<T, dfloat>::value>(d.Lz, [&](auto eng) {
         using F = decltype(eng);
+        if constexpr (std::is_same<T, double>::value) {
+            if constexpr (F::INPLACE) {
+                constexpr int A = F::A_, B = F::B_, TXC = F::TPL < 8 ? 16 : 4, NL = 3 * TXC;
+                constexpr int YB = B * fft4_ystride<A, fxc>(NL);
+                const size_t smf = (size_t)(YB > A * B * NL ? YB : A * B * NL) * sizeof(fxc) + (size_t)A * B * TXC * sizeof(int);
+                smem_attr((const void*)k4_fftz_green_fx<CONJ, A, B, TXC>, smf, FX_STATIC_SM);
+                k4_fftz_green_fx<CONJ, A, B, TXC><<<dim3(cdiv(d.Lx, TXC) * nsys, d.Ly, 1), NL * F::TPL, smf, st>>>(
+                    d, fx_twostep(pl, 2, A * B), sys, nsys, in_count, in_off, out_count, out_off, src_sel, dst_sel,
+                    fx_bits(A * B, in_count, A / 2 + 1, B), fx_bits(A * B, A * B, A, B));
+            } else {
+                with_width(fxg_width(d.Lz, 3, d.Lz > 128 ? 2 : 4, SMEM_CAP, v), [&](auto w) {
+                    constexpr int TXC = decltype(w)::value, NL = 3 * TXC;
+                    const size_t smf = (size_t)d.Lz * (2 * NL * sizeof(fxc) + TXC * sizeof(int));
+                    const int m = fxg_groups(pl.pz, 8, NL < 8 ? 32 : 192 / NL);
+                    smem_attr((const void*)kg_fftz_green_fx<CONJ, TXC>, smf, FX_STATIC_SM);
+                    kg_fftz_green_fx<CONJ, TXC><<<dim3(cdiv(d.Lx, TXC) * nsys, d.Ly, 1), NL * m, smf, st>>>(
+                        d, pl.pz, fx_tables(pl, 2), sys, nsys, in_count, in_off, out_count, out_off, src_sel, dst_sel);
+                });
+            }
+        } else {
         int TX, th;
         size_t sm;
         strided_cfg<T, F>(d.Lz, 3, TX, th, sm, v == 2);
@@ -1546,15 +1628,7 @@ static void launch_zpass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
             return;
           }
         }
-        if constexpr (F::INPLACE && std::is_same<T, double>::value) {
-            constexpr int A = F::A_, B = F::B_, TXC = F::TPL < 8 ? 16 : 4, NL = 3 * TXC;
-            constexpr int YB = B * fft4_ystride<A, fxc>(NL);
-            const size_t smf = (size_t)(YB > A * B * NL ? YB : A * B * NL) * sizeof(fxc) + (size_t)A * B * TXC * sizeof(int);
-            smem_attr((const void*)k4_fftz_green_fx<CONJ, A, B, TXC>, smf);
-            k4_fftz_green_fx<CONJ, A, B, TXC><<<dim3(cdiv(d.Lx, TXC) * nsys, d.Ly, 1), NL * F::TPL, smf, st>>>(
-                d, pl.fxz, sys, nsys, in_count, in_off, out_count, out_off, src_sel, dst_sel, fx_bits(A * B, in_count, A / 2 + 1, B),
-                fx_bits(A * B, A * B, A, B));
-        } else if constexpr (F::INPLACE) {
+        if constexpr (F::INPLACE) {
             constexpr int A = F::A_, B = F::B_, TXC = 4;
             smem_attr((const void*)k4_fftz_green<T, CONJ, A, B, TXC>, sm);
             k4_fftz_green<T, CONJ, A, B, TXC><<<dim3(cdiv(d.Lx, TXC), d.Ly, 1), th, sm, st>>>(
@@ -1563,6 +1637,7 @@ static void launch_zpass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
             smem_attr((const void*)k_fftz_green<T, CONJ, F>, sm);
             k_fftz_green<T, CONJ, F><<<dim3(cdiv(d.Lx, TX), d.Ly, nsys), th, sm, st>>>(
                 d, pl.pz, (const C*)pl.twz, sys, TX, in_count, in_off, out_count, out_off, src_sel, dst_sel);
+        }
         }
     }, v);
 }
@@ -1659,7 +1734,7 @@ static cudaError_t launch_apply_h(const Medium& m, const Plans& pl, const ApplyS
     ktimer_mark(tm, 0, f32, st, 1);
     // 2. forward x FFT of the 9 planes: w1 -> w2 [9][nz][ny][Lx]
     ktimer_mark(tm, 1, f32, st, 0);
-    launch_xrows<T>(d, sys, nsys, pl, 2, 3, 9LL * d.nz * d.ny, d.nx, st);
+    launch_xrows<T, -1>(d, sys, nsys, pl, 2, 3, 9LL * d.nz * d.ny, d.nx, 0, d.Lx, 0, st);
     ktimer_mark(tm, 1, f32, st, 1);
     // 3. forward y FFT: w2 -> w1 [9][nz][Ly][Lx]
     ktimer_mark(tm, 2, f32, st, 0);
@@ -1746,17 +1821,9 @@ cudaError_t launch_apply(const Medium& m, const Plans& pl, const ApplySys<T>* sy
 // z = K_T^H u on the extended nodes, left in w1 [3][ez][ey][ex] (the first five steps of A^H).
 template <typename T>
 static void launch_adjoint_conv(const Medium& m, const Plans& pl, const ApplySys<T>* sys, int nsys, cudaStream_t st) {
-    typedef typename cplx_of<T>::type C;
     const Dims& d = m.d;
-    const C* twx = (const C*)pl.twx;
     // 1. w placed at x positions 1..nx, forward x FFT: u [3][nz][ny][nx] -> w1 [3][nz][ny][Lx]
-    {
-        const int NL = generic_rows_nl<T>(d.Lx);
-        const long long nrows = 3LL * d.nz * d.ny;
-        const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(C);
-        smem_attr((const void*)k_rows<T, -1>, sm);
-        k_rows<T, -1><<<dim3(cdiv(nrows, NL), nsys), NTH, sm, st>>>(pl.px, twx, sys, 0, 2, nrows, NL, d.nx, 1, d.Lx, 0);
-    }
+    launch_xrows<T, -1>(d, sys, nsys, pl, 0, 2, 3LL * d.nz * d.ny, d.nx, 1, d.Lx, 0, st, std::is_same<T, double>::value ? 0 : 1);
     // 2. forward y FFT, input at 1..ny: w1 [3][nz][ny][Lx] -> w2 [3][nz][Ly][Lx]
     launch_ypass<T, -1>(d, sys, nsys, pl, d.nz, d.ny, 1, d.Ly, 0, 2, 3, st);
     // 3. z: input at 1..nz, conj(G-hat), output extended 0..ez-1: w2 -> w1 [3][ez][Ly][Lx]
@@ -1764,13 +1831,7 @@ static void launch_adjoint_conv(const Medium& m, const Plans& pl, const ApplySys
     // 4. inverse y FFT, keep 0..ey-1: w1 [3][ez][Ly][Lx] -> w2 [3][ez][ey][Lx]
     launch_ypass<T, 1>(d, sys, nsys, pl, d.ez, d.Ly, 0, d.ey, 0, 2, 3, st);
     // 5. inverse x FFT, keep 0..ex-1: w2 [3][ez][ey][Lx] -> w1 [3][ez][ey][ex]
-    {
-        const int NL = generic_rows_nl<T>(d.Lx);
-        const long long nrows = 3LL * d.ez * d.ey;
-        const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(C);
-        smem_attr((const void*)k_rows<T, 1>, sm);
-        k_rows<T, 1><<<dim3(cdiv(nrows, NL), nsys), NTH, sm, st>>>(pl.px, twx, sys, 3, 2, nrows, NL, d.Lx, 0, d.ex, 0);
-    }
+    launch_xrows<T, 1>(d, sys, nsys, pl, 3, 2, 3LL * d.ez * d.ey, d.Lx, 0, d.ex, 0, st, std::is_same<T, double>::value ? 0 : 1);
 }
 
 template <typename T>

@@ -111,14 +111,17 @@ __device__ __forceinline__ void fx_row(double2 (&in)[FourStep<A, B>::I1][NZ], fx
     }
 }
 
-// forward x FFT of zero-padded rows: row r of src (in_count elements, the rest zero) -> row r of dst
-template <int A, int B, int LPB>
+// x FFT of contiguous rows: row r of src holds in_count elements (placed at in_off; forward: the rest
+// of the line is zero), row r of dst receives outputs out_off .. out_off + out_count - 1 (inverse: the
+// first half and a little, as cropped lines have)
+template <int DIR, int A, int B, int LPB>
 __global__ void __launch_bounds__(LPB * FourStep<A LSM_COMMA B>::TPL, B == 32 ? 2 : 4) k4_rows_fx(const int4* __restrict__ tw,
                                                                             const ApplySys<double>* __restrict__ sys,
                                                                             int src_sel, int dst_sel, long long nrows,
-                                                                            int in_count, int bits) {
+                                                                            int in_count, int in_off, int out_count,
+                                                                            int out_off, int bits) {
     typedef FourStep<A, B> F;
-    constexpr int L = A * B, NZ = FxStep<A, B>::NZI;
+    constexpr int NZ = DIR < 0 ? FxStep<A, B>::NZI : A, NO = DIR > 0 ? FxStep<A, B>::NOO : B;
     static_assert(LPB * F::TPL % 32 == 0, "whole warps");
     extern __shared__ unsigned char smem_raw[];
     const ApplySys<double> S = sys[blockIdx.y];
@@ -127,18 +130,19 @@ __global__ void __launch_bounds__(LPB * FourStep<A LSM_COMMA B>::TPL, B == 32 ? 
     const long long row = (long long)blockIdx.x * LPB + ln;
     const bool live = row < nrows;
     const double2* __restrict__ src = pick<double2>(S, src_sel) + row * in_count;
-    double2* __restrict__ dst = pick<double2>(S, dst_sel) + row * L;
+    double2* __restrict__ dst = pick<double2>(S, dst_sel) + row * out_count;
     double2 in[F::I1][NZ];
 #pragma unroll
     for (int i = 0; i < F::I1; ++i)
 #pragma unroll
         for (int k = 0; k < NZ; ++k) {
-            const int e = q + F::TPL * i + B * k;
-            in[i][k] = (live && e < in_count) ? src[e] : czero<double2>();
+            const int e = q + F::TPL * i + B * k - in_off;
+            in[i][k] = (live && e >= 0 && e < in_count) ? src[e] : czero<double2>();
         }
     fxc* tl = reinterpret_cast<fxc*>(smem_raw) + ln * B * (A + 1);
-    fx_row<-1, A, B, NZ, B>(in, tl, tw, q, bits, [&](int k, double2 r) {
-        if (live) dst[k] = r;
+    fx_row<DIR, A, B, NZ, NO>(in, tl, tw, q, bits, [&](int k, double2 r) {
+        const int e = k - out_off;
+        if (live && e >= 0 && e < out_count) dst[e] = r;
     });
 }
 

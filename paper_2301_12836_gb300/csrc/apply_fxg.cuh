@@ -1,0 +1,308 @@
+// apply_fxg.cuh - the FP64 operator's transform passes in 64-bit fixed point (fx.cuh) for any line
+// length with factors 2, 3 and 5 (and for the two-step lengths on request of the schedule).
+// Included by apply.cu after apply_fx.cuh.
+//
+// Runtime mixed-radix Stockham stages (fft.cuh) between two shared-memory buffers.  A thread keeps
+// one line (l) and one of m groups of butterflies (g), so no stage divides by the tile's width; m is
+// chosen on the host so that the groups fill every stage's butterflies as evenly as they can
+// (fxg_groups).  Every stage after the first carries 2^-K in its twiddles, K = 1 .. 3 such that all
+// stages keep the same range (chosen with the plan): a line's error is that of its last stages (K = 2
+// or 3 by the radix alone lost up to 3 bits on lines such as 250 = 2 5 5 5: error 1.6 of the FP64
+// engine's, now 0.9 to 0.99).
+//
+// Bound by latency and the integer pipes (z pass at 96^3: issue 31% at 10 warps before the tile was
+// halved).  One system, FP64 apply: 96^3 4.62 -> 1.44 ms (z pass 2.74 -> 0.65, y 0.51 -> 0.14 each, inverse x
+// 0.30 -> 0.12), 60 x 45 x 50 0.92 -> 0.30 ms.
+#pragma once
+
+namespace lsm {
+
+// the two scaled twiddle tables of a line length: entries times 2^-2 and 2^-3
+struct FxTables {
+    const int4 *t2, *t3;
+};
+
+template <int S, int R, int LD>
+__device__ __forceinline__ void fxg_stage(const fxc* __restrict__ src, fxc* __restrict__ dst, int L, int Ns, int K,
+                                          const FxTables& T, int l, int g, int m) {
+    const int4* __restrict__ tw = K == 3 ? T.t3 : T.t2;
+    const int nb = L / R, tstep = L / (Ns * R);
+    const unsigned magic = 0xffffffffu / (unsigned)Ns + 1;   // j / Ns = j magic 2^-32 for j < 2^16 (Ns > 1)
+#pragma unroll 1
+    for (int j = g; j < nb; j += m) {
+        const int jq = Ns == 1 ? j : (int)__umulhi((unsigned)j, magic);
+        const int k = j - jq * Ns;
+        fxc v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = src[(j + r * nb) * LD + l];
+        if (K) {   // not the first stage
+            v[0].x = fx_r((fx_ll(v[0].x) + (1 << (K - 1))) >> K);
+            v[0].y = fx_r((fx_ll(v[0].y) + (1 << (K - 1))) >> K);
+#pragma unroll
+            for (int r = 1; r < R; ++r) {
+                if (K == 1) v[r] = cadd(v[r], v[r]);
+                v[r] = tw_mul32<S>(v[r], tw, r * k * tstep);
+            }
+        }
+        if constexpr (R == 2) bfly2<S>(v);
+        else if constexpr (R == 3) bfly3<S>(v);
+        else if constexpr (R == 4) bfly4<S>(v);
+        else if constexpr (R == 5) bfly5<S>(v);
+        else bfly8<S>(v);
+        const int base = jq * Ns * R + k;
+#pragma unroll
+        for (int r = 0; r < R; ++r) dst[(base + r * Ns) * LD + l] = v[r];
+    }
+}
+
+// Transform the tile in a (layout a[e * LD + l]); b is scratch of the same size.  Returns the buffer
+// of the result.  The caller synchronises before; the result is visible to the block on return.
+template <int S, int LD>
+__device__ __forceinline__ fxc* fxg_fft(fxc* a, fxc* b, const FftPlan& p, const FxTables& T, int l, int g, int m) {
+    int Ns = 1;
+    for (int s = 0; s < p.nst; ++s) {
+        const int R = p.radix[s];
+        switch (R) {
+            case 8: fxg_stage<S, 8, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
+            case 4: fxg_stage<S, 4, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
+            case 2: fxg_stage<S, 2, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
+            case 3: fxg_stage<S, 3, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
+            default: fxg_stage<S, 5, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
+        }
+        __syncthreads();
+        fxc* t = a; a = b; b = t;
+        Ns *= R;
+    }
+    return a;
+}
+
+// Groups per line, m <= most: the fewest butterfly rounds weighted by their size, then the most groups.
+static inline int fxg_groups(const FftPlan& p, int least, int most) {
+    int best = least;
+    double cost = 1e300;
+    for (int m = least; m <= most; ++m) {
+        double c = 0.0;
+        for (int s = 0; s < p.nst; ++s) {
+            const int nb = p.L / p.radix[s];
+            c += (double)((nb + m - 1) / m) * (p.radix[s] + 2) * m;
+        }
+        c *= 1.0 + 4.0 / m;   // fewer threads hide less latency
+        if (c <= cost) {
+            cost = c;
+            best = m;
+        }
+    }
+    return best;
+}
+
+// Elements g, g + m, ... below n of a line, ld(e) -> raw[e * LD + l], four loads in flight; returns the
+// largest magnitude word.
+template <int LD, class Ld>
+__device__ __forceinline__ unsigned fxg_load(double2* raw, int n, int l, int g, int m, Ld ld) {
+    unsigned mag = 0;
+    for (int e = g; e < n; e += 4 * m) {
+        double2 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = e + k * m < n ? ld(e + k * m) : czero<double2>();
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (e + k * m < n) {
+                raw[(e + k * m) * LD + l] = v[k];
+                mag = max(mag, max(fx_mag(v[k].x), fx_mag(v[k].y)));
+            }
+    }
+    return mag;
+}
+
+// ---- strided pass: NL consecutive lines along x per block
+template <int DIR, int NL>
+__global__ void __launch_bounds__(NL * 48) kg_strided_fx(FftPlan p, FxTables T, StridedArgs a, const ApplySys<double>* __restrict__ sys) {
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ unsigned s_mag[NL];
+    const ApplySys<double>& S = sys[blockIdx.z / a.ncomp];
+    if (S.run && !*S.run) return;
+    const int c = blockIdx.z % a.ncomp;
+    const int l = threadIdx.x % NL, g = threadIdx.x / NL, m = blockDim.x / NL;
+    const int x = blockIdx.x * NL + l;
+    const bool xin = x < a.nlines;
+    const double2* __restrict__ src = pick<double2>(S, a.src_sel) + c * a.src_os2 + blockIdx.y * a.src_os1 + x;
+    double2* __restrict__ dst = pick<double2>(S, a.dst_sel) + c * a.dst_os2 + blockIdx.y * a.dst_os1 + x;
+    fxc* sa = reinterpret_cast<fxc*>(smem_raw);
+    fxc* sb = sa + (size_t)p.L * NL;
+    double2* raw = reinterpret_cast<double2*>(sb);
+    if (threadIdx.x < NL) s_mag[threadIdx.x] = 0;
+    __syncthreads();
+    const unsigned mag = fxg_load<NL>(raw, a.in_count, l, g, m, [&](int e) { return xin ? src[(long long)e * a.src_es] : czero<double2>(); });
+    atomicMax(&s_mag[l], mag);
+    __syncthreads();
+    const FxScale sc(s_mag[l]);
+    for (int e = g; e < p.L; e += m) {
+        const int es = e - a.in_off;
+        sa[e * NL + l] = (es >= 0 && es < a.in_count) ? fx_from(raw[es * NL + l], sc, p.fxbits) : czero<fxc>();
+    }
+    __syncthreads();
+    const fxc* r = fxg_fft<DIR, NL>(sa, sb, p, T, l, g, m);
+    const FxUnit un(sc.unit(p.fxbits) + p.fxsum, sc.bad, s_mag[l] == 0);
+    if (xin)
+        for (int eo = g; eo < a.out_count; eo += m) {
+            const fxc v = r[(eo + a.out_off) * NL + l];
+            dst[(long long)eo * a.dst_es] = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
+        }
+}
+
+// ---- contiguous rows: NL rows per block.  Row r of src holds in_count elements (placed at in_off),
+// row r of dst out_count (from out_off).  OUT: the inverse x pass's epilogue, dst = S.out = u - result.
+template <int DIR, int NL, bool OUT>
+__global__ void __launch_bounds__(NL * 48) kg_rows_fx(FftPlan p, FxTables T, const ApplySys<double>* __restrict__ sys, int src_sel,
+                                                      int dst_sel, long long nrows, int in_count, int in_off, int out_count,
+                                                      int out_off) {
+    constexpr int LD = NL + 1;
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ unsigned s_mag[NL];
+    const ApplySys<double>& S = sys[blockIdx.y];
+    if (S.run && !*S.run) return;
+    const int l = threadIdx.x % NL, g = threadIdx.x / NL, m = blockDim.x / NL;
+    const long long r0 = (long long)blockIdx.x * NL;
+    const int live = nrows - r0 < NL ? (int)(nrows - r0) : NL;
+    const double2* __restrict__ src = pick<double2>(S, src_sel) + r0 * in_count;
+    double2* __restrict__ dst = (OUT ? S.out : pick<double2>(S, dst_sel)) + r0 * out_count;
+    const double2* __restrict__ uin = OUT ? S.u + r0 * out_count : nullptr;
+    fxc* sa = reinterpret_cast<fxc*>(smem_raw);
+    fxc* sb = sa + (size_t)p.L * LD;
+    double2* raw = reinterpret_cast<double2*>(sb);
+    if (threadIdx.x < NL) s_mag[threadIdx.x] = 0;
+    __syncthreads();
+    for (int k = 0; k < live; ++k) {
+        unsigned mag = 0;
+        for (int e = threadIdx.x; e < in_count; e += blockDim.x) {
+            const double2 v = src[(long long)k * in_count + e];
+            raw[e * LD + k] = v;
+            mag = max(mag, max(fx_mag(v.x), fx_mag(v.y)));
+        }
+        if (mag) atomicMax(&s_mag[k], mag);
+    }
+    __syncthreads();
+    const FxScale sc(s_mag[l]);
+    for (int e = g; e < p.L; e += m) {
+        const int es = e - in_off;
+        sa[e * LD + l] = (l < live && es >= 0 && es < in_count) ? fx_from(raw[es * LD + l], sc, p.fxbits) : czero<fxc>();
+    }
+    __syncthreads();
+    const fxc* r = fxg_fft<DIR, LD>(sa, sb, p, T, l, g, m);
+    for (int k = 0; k < live; ++k) {
+        const FxScale sk(s_mag[k]);
+        const FxUnit un(sk.unit(p.fxbits) + p.fxsum, sk.bad, s_mag[k] == 0);
+        for (int e = threadIdx.x; e < out_count; e += blockDim.x) {
+            const fxc v = r[(e + out_off) * LD + k];
+            const double2 w = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
+            const long long i = (long long)k * out_count + e;
+            dst[i] = OUT ? csub(uin[i], w) : w;
+        }
+    }
+    if (OUT && S.count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(S.count, 1ull);
+}
+
+// ---- z pass with the Green multiply: TX columns of one ky, as k4_fftz_green_fx
+template <bool CONJ, int TX>
+__global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FftPlan p, FxTables T, const ApplySys<double>* __restrict__ sys,
+                                                                int nsys, int in_count, int in_off, int out_count, int out_off,
+                                                                int src_sel, int dst_sel) {
+    constexpr int NL = 3 * TX;
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ unsigned s_mag[TX];
+    __shared__ int s_key[TX];
+    const ApplySys<double>& S = sys[blockIdx.x % nsys];
+    if (S.run && !*S.run) return;
+    const int L = p.L;
+    const int x0 = (int)(blockIdx.x / nsys) * TX, ky = blockIdx.y;
+    const int l = threadIdx.x % NL, g = threadIdx.x / NL, m = blockDim.x / NL;
+    const int cl = l / TX, lx = l - cl * TX;
+    const bool xin = x0 + lx < d.Lx;
+    const unsigned plane = (unsigned)(d.Ly * d.Lx), col = (unsigned)(ky * d.Lx + x0 + lx);
+    fxc* sa = reinterpret_cast<fxc*>(smem_raw);
+    fxc* sb = sa + (size_t)L * NL;
+    int* sE = reinterpret_cast<int*>(sb + (size_t)L * NL);   // [L][TX]
+    double2* raw = reinterpret_cast<double2*>(sb);
+    if (threadIdx.x < TX) {
+        s_mag[threadIdx.x] = 0;
+        s_key[threadIdx.x] = FX_NO_KEY;
+    }
+    __syncthreads();
+    {
+        const double2* __restrict__ src = pick<double2>(S, src_sel) + (size_t)cl * in_count * plane + col;
+        const unsigned mag = fxg_load<NL>(raw, in_count, l, g, m, [&](int e) { return xin ? src[(size_t)e * plane] : czero<double2>(); });
+        atomicMax(&s_mag[lx], mag);
+    }
+    __syncthreads();
+    const FxScale sc(s_mag[lx]);
+    for (int e = g; e < L; e += m) {
+        const int es = e - in_off;
+        sa[e * NL + l] = (es >= 0 && es < in_count) ? fx_from(raw[es * NL + l], sc, p.fxbits) : czero<fxc>();
+    }
+    __syncthreads();
+    fxc* s = fxg_fft<-1, NL>(sa, sb, p, T, l, g, m);
+    fxc* o = s == sa ? sb : sa;
+    // ---- Green multiply
+    {
+        const int cx = threadIdx.x % TX, kx = x0 + cx;   // blockDim.x is a multiple of TX
+        int key = FX_NO_KEY;
+        if (kx < d.Lx) {
+            const long long NO = (long long)(d.nx + 1) * (d.ny + 1) * (d.nz + 1);
+            const int fy = ky <= d.ny ? ky : d.Ly - ky, fx = kx <= d.nx ? kx : d.Lx - kx;
+            const int sgx = kx > d.nx ? -1 : 1, sgy = ky > d.ny ? -1 : 1;
+            const unsigned o0 = (unsigned)(fy * (d.nx + 1) + fx), oz = (unsigned)((d.nx + 1) * (d.ny + 1));
+            const int4* __restrict__ gx = S.gx;
+            const int* __restrict__ gexp = S.ge;
+            const int dk = blockDim.x / TX;
+            int4 G[6];
+            int ge = 0;
+            auto fetch = [&](int k) {
+                const unsigned w = (unsigned)(k <= d.nz ? k : L - k) * oz + o0;
+#pragma unroll
+                for (int c = 0; c < 6; ++c) G[c] = __ldg(gx + c * NO + w);
+                ge = __ldg(gexp + w);
+            };
+            int kz = threadIdx.x / TX;
+            if (kz < L) fetch(kz);
+#pragma unroll 1
+            for (; kz < L; kz += dk) {
+                const int sgz = kz > d.nz ? -1 : 1;
+                const int4 G0 = G[0], G1 = G[1], G2 = G[2];
+                const int4 G3 = fx_flip(G[3], sgy * sgz), G4 = fx_flip(G[4], sgx * sgz), G5 = fx_flip(G[5], sgx * sgy);
+                const int e = ge;
+                if (kz + dk < L) fetch(kz + dk);   // in flight during this point's products
+                fxc* row = s + kz * NL + cx;
+                const FxQ qa(row[0]), qb(row[TX]), qc(row[2 * TX]);
+                const fxc r0 = fx_gdot3<CONJ>(G0, qa, G5, qb, G4, qc);
+                row[0] = r0;
+                const fxc r1 = fx_gdot3<CONJ>(G5, qa, G1, qb, G3, qc);
+                row[TX] = r1;
+                const fxc r2 = fx_gdot3<CONJ>(G4, qa, G3, qb, G2, qc);
+                row[2 * TX] = r2;
+                sE[kz * TX + cx] = e;
+                key = max(key, 64 - __clz((int)(fx_hibits(r0) | fx_hibits(r1) | fx_hibits(r2))) + e);
+            }
+            atomicMax(&s_key[cx], key);
+        }
+        __syncthreads();
+    }
+    // ---- inverse transform
+    const int top = s_key[lx], ecom = top - p.fxbits;
+    for (int e = g; e < L; e += m) {
+        fxc v = s[e * NL + l];
+        const int sh = ecom - (xin ? sE[e * TX + lx] : 0);
+        s[e * NL + l] = fxc{fx_shift(v.x, sh), fx_shift(v.y, sh)};
+    }
+    __syncthreads();
+    const fxc* r = fxg_fft<1, NL>(s, o, p, T, l, g, m);
+    const FxUnit un(sc.unit(p.fxbits) + 2 * p.fxsum + ecom, sc.bad || top > FxG::BAD_EXP / 2, s_mag[lx] == 0);
+    if (xin) {
+        double2* __restrict__ dst = pick<double2>(S, dst_sel) + (size_t)cl * out_count * plane + col;
+        for (int eo = g; eo < out_count; eo += m) {
+            const fxc v = r[(eo + out_off) * NL + l];
+            dst[(size_t)eo * plane] = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
+        }
+    }
+}
+
+}  // namespace lsm

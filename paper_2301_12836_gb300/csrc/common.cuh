@@ -130,6 +130,10 @@ struct FftPlan {
     int L;
     int nst;
     int radix[12];
+    // fixed-point runs of the plan (apply_fxg.cuh): K of each stage, bits of the inputs, and the sum
+    // of the K by which the outputs' unit is coarser than the inputs'
+    int fxk[12];
+    int fxbits, fxsum;
 };
 
 }  // namespace lsm

@@ -149,6 +149,11 @@ __device__ __forceinline__ fxc fx_cmul32(fxc a, int r1, int r0, int i1, int i0) 
     const fxr ti = fx_words(fx_mad(yh, r0, fx_mad(yl, r1, fx_mad(xh, i0, fx_mad(xl, i1, 1LL << 31)))));
     return fxc{fx_words(fx_mad(yh, -i1, fx_mad(xh, r1, fx_sext(tr.h)))), fx_words(fx_mad(yh, r1, fx_mad(xh, i1, fx_sext(ti.h))))};
 }
+// v 2^-sh, rounded to nearest, for sh of either sign; 64 or more shifts any value out
+__device__ __forceinline__ fxr fx_shift(fxr v, int sh) {
+    if (sh > 0) return fx_r(((fx_ll(v) >> min(sh - 1, 62)) + 1) >> 1);
+    return fx_r((long long)((unsigned long long)fx_ll(v) << min(-sh, 63)));
+}
 // +-a +-b
 __device__ __forceinline__ fxr fx_pm(fxr a, bool pa, fxr b, bool pb) {
     return pa ? (pb ? fx_add(a, b) : fx_sub(a, b)) : (pb ? fx_sub(b, a) : fx_neg(fx_add(a, b)));
@@ -166,15 +171,11 @@ template <int S> __device__ __forceinline__ fxc cmul_const(fxc a, double re, dou
 }
 
 // a tw[k] (S < 0) or a conj(tw[k]) (S > 0); a fixed-point entry is (W1, W0) of the real part, then
-// of the imaginary part, in the two forms of fx_cmul32 (the two-step plans) and fx_cmul
+// of the imaginary part, scaled for fx_cmul32
 template <int S, typename C> __device__ __forceinline__ C tw_mul(C a, const C* __restrict__ tw, int k) {
     C w = __ldg(&tw[k]);
     if (S > 0) w.y = -w.y;
     return cmul(a, w);
-}
-template <int S> __device__ __forceinline__ fxc tw_mul(fxc a, const int4* __restrict__ tw, int k) {
-    const int4 w = __ldg(&tw[k]);
-    return S > 0 ? fx_cmul(a, w.x, w.y, -w.z, -w.w) : fx_cmul(a, w.x, w.y, w.z, w.w);
 }
 template <int S> __device__ __forceinline__ fxc tw_mul32(fxc a, const int4* __restrict__ tw, int k) {
     // volatile: 15 entries fetched ahead of their use would spill
@@ -182,11 +183,8 @@ template <int S> __device__ __forceinline__ fxc tw_mul32(fxc a, const int4* __re
     asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(tw + k));
     return S > 0 ? fx_cmul32(a, w.x, w.y, -w.z, -w.w) : fx_cmul32(a, w.x, w.y, w.z, w.w);
 }
-// K of the two-step plan of length L; 0 for the lengths of the generic engine, whose transforms keep
-// one unit and plain twiddles.
-__host__ __device__ constexpr int fx_prescale(int L) {
-    return L == 16 ? 2 : (L == 32 || L == 64 || L == 128 || L == 256 || L == 512 ? 3 : 0);
-}
+// K of the two-step plan of length L
+__host__ __device__ constexpr int fx_prescale(int L) { return L == 16 ? 2 : 3; }
 
 // twiddles between the steps of a two-step transform of length L: v[k1] tw[t k1].  Row t = 0 has
 // none; in fixed point every entry also passes to the second step's unit (the table's entries carry
@@ -284,13 +282,13 @@ __device__ __forceinline__ double2 fx_to_odd(fxc v, const FxUnit& u) { return ma
 // Bits of a line's inputs, in the unit of the outputs: a line with at most nin nonzero inputs, each
 // component below 2^bits in modulus, keeps its outputs below 2^62.6 (log2(nin) + 1/2 bits of growth).
 // last: radix of the last step's DFT; 8 and 32 multiply just before their final additions, so one
-// bit less keeps those products' factors in range; generic plans (last = 0) likewise.  nz: nonzero
+// bit less keeps those products' factors in range.  nz: nonzero
 // inputs of a first-step DFT, whose outputs, 2^K finer, stay below 2^61.9.
 inline int fx_bits(int L, int nin, int nz, int last) {
     const double one = 4611686018427387904.0;   // 2^62
     int b = 62;
     while (b > 0 && (double)nin * (double)(1ull << b) > 1.0717734625362931 * one) --b;   // 2^62.1
-    if (last == 8 || last == 32 || last == 0) --b;
+    if (last == 8 || last == 32) --b;
     while (b > 0 && (double)nz * (double)(1ull << b) * (1 << fx_prescale(L)) > 0.6597539553864471 * one) --b;   // 2^61.4
     return b;
 }

@@ -56,8 +56,8 @@ struct Plans {
     const void* twx;     // twiddle tables of T: exp(-2 pi i k / L)
     const void* twy;
     const void* twz;
-    // FP64 plans: the same tables as two-word fixed-point numbers (fx.cuh)
-    const int4 *fxx = nullptr, *fxy = nullptr, *fxz = nullptr;
+    // FP64 plans: the same tables as two-word fixed-point numbers scaled by 2^-2 and 2^-3 (fx.cuh)
+    const int4 *fx2[3] = {nullptr, nullptr, nullptr}, *fx3[3] = {nullptr, nullptr, nullptr};
 };
 
 // workspace elements (complex) needed by one system's apply / adjoint in w1 and w2 (kernel as in Medium)

@@ -118,7 +118,7 @@ struct lsm_ctx {
     lsm_opts o;
     double2* ghat64 = nullptr;
     int4* gx = nullptr;       // fixed-point copy of the G spectra for the FP64 z pass, and ...
-    int* ge = nullptr;        // ... its exponent per point
+    int* ge = nullptr;        // ... its exponent per point (in gx's allocation)
     float2* ghat32 = nullptr;
     dfcplx* ghatdf = nullptr;
     long long nl = 0;
@@ -143,6 +143,25 @@ lsm_status cuda_fail(lsm_t h, cudaError_t e, const char* where) {
         if (_e != cudaSuccess) return cuda_fail(h, _e, #call); \
     } while (0)
 
+// Scaling of a plan's fixed-point stages: in log2 of the largest modulus, the first stage's outputs and
+// every later stage's stay below 61.9 with the smallest K in 1 .. 3 that does it (K = 1 doubles the
+// values before a product, which needs them below 60.9).
+void fixed_point_scaling(FftPlan& p) {
+    const double top = 61.9;
+    const double g0 = log2((double)p.radix[0]);
+    p.fxbits = (int)floor(top - 0.5 - g0);
+    double m = p.fxbits + 0.5 + g0;
+    p.fxk[0] = 0;
+    p.fxsum = 0;
+    for (int s = 1; s < p.nst; ++s) {
+        const double g = log2((double)p.radix[s]);
+        int k = (m <= top - 1.0 && m + g - 1.0 <= top) ? 1 : (m + g - 2.0 <= top ? 2 : 3);
+        p.fxk[s] = k;
+        p.fxsum += k;
+        m += g - k;
+    }
+}
+
 bool factor_plan(int L, FftPlan& p) {
     p.L = L;
     p.nst = 0;
@@ -155,37 +174,36 @@ bool factor_plan(int L, FftPlan& p) {
             m /= rs[k];
         }
     }
+    if (m == 1) fixed_point_scaling(p);
     return m == 1;
 }
 
-// v (|v| <= 1) as the two-word fixed-point number v1 2^-w + v0 2^-2w, both words within
-// +-(2^31 - 1) so that either sign can be negated
-void fx_words(long double v, int w, int* v1, int* v0) {
-    const long double lim = 2147483647.0L, f = (long double)(1LL << w);
-    long double a = nearbyintl(v * f);
-    a = a > lim ? lim : (a < -lim ? -lim : a);
-    long double b = nearbyintl((v * f - a) * f);
-    b = b > lim ? lim : (b < -lim ? -lim : b);
+// v (|v| <= 1/4) as the two-word fixed-point number v1 2^-32 + v0 2^-64, v0 within +-(2^31 - 1) so
+// that either sign can be negated
+void fx_table_words(long double v, int* v1, int* v0) {
+    const long double f = 4294967296.0L, lim = 2147483647.0L;
+    const long double a = nearbyintl(v * f);
+    const long double b = nearbyintl((v * f - a) * f);
     *v1 = (int)a;
-    *v0 = (int)b;
+    *v0 = (int)(b > lim ? lim : (b < -lim ? -lim : b));
 }
 
-// exp(-2 pi i k / L), k < L, evaluated in long double and rounded once (the fixed-point table with
-// the two-step transforms' change of unit, fx.cuh)
-void twiddle_table(int L, std::vector<double2>& t64, std::vector<float2>& t32, std::vector<int4>& tfx) {
+// exp(-2 pi i k / L), k < L, evaluated in long double and rounded once; fx2, fx3: as fixed-point words
+// times 2^-2 and 2^-3
+void twiddle_table(int L, std::vector<double2>& t64, std::vector<float2>& t32, std::vector<int4>& fx2, std::vector<int4>& fx3) {
     const long double pi = 3.141592653589793238462643383279502884L;
     for (int k = 0; k < L; ++k) {
         const long double a = -2.0L * pi * (long double)k / (long double)L;
         const long double c = cosl(a), s = sinl(a);
         t64.push_back(make_double2((double)c, (double)s));
         t32.push_back(make_float2((float)c, (float)s));
-        // two-step plans: scaled to below 1/2, split at the words (fx_cmul32); generic plans: fx_cmul
-        const int K = fx_prescale(L);
-        const long double f = 1.0L / (1 << K);
         int4 w;
-        fx_words(c * f, K ? 32 : 31, &w.x, &w.y);
-        fx_words(s * f, K ? 32 : 31, &w.z, &w.w);
-        tfx.push_back(w);
+        fx_table_words(c / 4, &w.x, &w.y);
+        fx_table_words(s / 4, &w.z, &w.w);
+        fx2.push_back(w);
+        fx_table_words(c / 8, &w.x, &w.y);
+        fx_table_words(s / 8, &w.z, &w.w);
+        fx3.push_back(w);
     }
 }
 
@@ -320,8 +338,8 @@ static lsm_status build_spectrum(lsm_t h) {
     cudaFree(scratch);
     if (e != cudaSuccess) return cuda_fail(h, e, "green spectrum setup");
     if (s->kernel == LSM_KERNEL_DIFF) {
-        CK(h, cudaMalloc(&h->gx, 6 * NO * sizeof(int4)));
-        CK(h, cudaMalloc(&h->ge, NO * sizeof(int)));
+        CK(h, cudaMalloc(&h->gx, 6 * NO * sizeof(int4) + NO * sizeof(int)));
+        h->ge = (int*)(h->gx + 6 * NO);
         CK(h, launch_fx_spectrum(h->ghat64, NO, h->gx, h->ge, s->st, &h->nl));
         CK(h, cudaStreamSynchronize(s->st));
     }
@@ -392,13 +410,19 @@ extern "C" lsm_status lsm_create(lsm_t* out, const int n[3], double dx, double l
         s->pl32.px = s->pl64.px; s->pl32.py = s->pl64.py; s->pl32.pz = s->pl64.pz;
         std::vector<double2> t64;
         std::vector<float2> t32;
-        std::vector<int4> tfx;
-        twiddle_table(d.Lx, t64, t32, tfx);
-        twiddle_table(d.Ly, t64, t32, tfx);
-        twiddle_table(d.Lz, t64, t32, tfx);
-        CKB(cudaMalloc(&s->twfx, tfx.size() * sizeof(int4)));
-        CKB(cudaMemcpy(s->twfx, tfx.data(), tfx.size() * sizeof(int4), cudaMemcpyHostToDevice));
-        s->pl64.fxx = s->twfx; s->pl64.fxy = s->twfx + d.Lx; s->pl64.fxz = s->twfx + d.Lx + d.Ly;
+        std::vector<int4> f2, f3;
+        twiddle_table(d.Lx, t64, t32, f2, f3);
+        twiddle_table(d.Ly, t64, t32, f2, f3);
+        twiddle_table(d.Lz, t64, t32, f2, f3);
+        const size_t nt = f2.size();
+        f2.insert(f2.end(), f3.begin(), f3.end());
+        CKB(cudaMalloc(&s->twfx, f2.size() * sizeof(int4)));
+        CKB(cudaMemcpy(s->twfx, f2.data(), f2.size() * sizeof(int4), cudaMemcpyHostToDevice));
+        const int off[3] = {0, d.Lx, d.Lx + d.Ly};
+        for (int a = 0; a < 3; ++a) {
+            s->pl64.fx2[a] = s->twfx + off[a];
+            s->pl64.fx3[a] = s->twfx + nt + off[a];
+        }
         CKB(cudaMalloc(&s->tw64, t64.size() * sizeof(double2)));
         CKB(cudaMalloc(&s->tw32, t32.size() * sizeof(float2)));
         CKB(cudaMemcpy(s->tw64, t64.data(), t64.size() * sizeof(double2), cudaMemcpyHostToDevice));
@@ -475,7 +499,6 @@ extern "C" void lsm_destroy(lsm_t h) {
     if (!h) return;
     cudaFree(h->ghat64);
     cudaFree(h->gx);
-    cudaFree(h->ge);
     cudaFree(h->ghat32);
     cudaFree(h->ghatdf);
     store_release(h->s);

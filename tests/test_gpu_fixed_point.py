@@ -69,3 +69,35 @@ def test_zero_infinite_and_nan_fields(n):
         v = u.copy()
         v[2, n[2] // 2, n[1] // 3, n[0] // 3] = bad
         assert np.all(np.isnan(_apply(h, v)))
+
+
+# generic lengths: every radix first and last, one-stage plans, the longest line, tile remainders
+GENERIC = [(2, 3, 4), (5, 6, 10), (9, 15, 25), (27, 12, 45), (50, 81, 6), (6, 125, 9), (10, 9, 125), (250, 3, 4), (4, 250, 3),
+           (3, 4, 250), (96, 5, 12), (5, 96, 4), (12, 5, 96)]
+
+
+@pytest.mark.parametrize("n", GENERIC)
+def test_generic_lengths(n):
+    """Forward and adjoint operators against the oracle, and the exact scaling, on lines of the
+    runtime engine."""
+    med = sy.random_medium(n, h=8.0, seed=sum(n) + 3, frac=0.2)
+    h = handle(med, W)
+    F = op.FFTOperator(med, W)
+    u = field(med.shape, 10)
+    got, got_h = _apply(h, u), _apply(h, u, True)
+    assert rel(got, F.apply(u)) < 1e-12
+    assert rel(got_h, F.adjoint(u)) < 1e-12
+    assert np.array_equal(_apply(h, u * 2.0 ** -500), got * 2.0 ** -500)
+    assert not np.any(_apply(h, np.zeros_like(u)))
+
+
+@pytest.mark.parametrize("v", [1, 2])
+def test_generic_engine_on_two_step_lengths(v):
+    """The schedule's generic variants of 16 .. 256: within rounding of the default kernels."""
+    for n in ((8, 16, 32), (64, 8, 8), (8, 9, 128)):
+        med = sy.random_medium(n, h=8.0, seed=sum(n) + 4, frac=0.2)
+        h = handle(med, W)
+        u = field(med.shape, 11)
+        want = _apply(h, u)
+        lsm.lsm_set_schedule(h, lsm.LSM_FP64, [0, v, v, v, v, v])
+        assert rel(_apply(h, u), want) < 2e-14
