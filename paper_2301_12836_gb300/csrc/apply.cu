@@ -1998,9 +1998,41 @@ cudaError_t fft3_inplace_setup(const Dims& d, const Plans& pl, double2* buf, int
     return cudaGetLastError();
 }
 
-cudaError_t launch_fx_spectrum(const double2* ghat64, long long NO, int4* gx, int* ge, cudaStream_t st, long long* nl) {
-    k_fx_spectrum<<<grid_elems(NO), NTH, 0, st>>>(ghat64, NO, gx, ge);
+cudaError_t launch_spectrum_forms(const double2* g, double scale, long long NO, int4* gx, int* ge, float2* g32, dfcplx* gdf,
+                                  cudaStream_t st, long long* nl) {
+    k_spectrum_forms<<<grid_elems(NO), NTH, 0, st>>>(g, scale, NO, gx, ge, g32, gdf);
     if (nl) *nl += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_octant_fft(const Dims& d, const Plans& pl, double2* buf, cudaStream_t st, long long* nl) {
+    const long long sx = d.nx + 1, sy = d.ny + 1, sz = d.nz + 1;
+    // components odd along each axis (order 11, 22, 33, 23, 13, 12)
+    const int odd[3] = {1 << 4 | 1 << 5, 1 << 3 | 1 << 5, 1 << 3 | 1 << 4};
+    const FftPlan* p[3] = {&pl.px, &pl.py, &pl.pz};
+    for (int a = 0; a < 3; ++a) {
+        SymArgs s;
+        s.cs = sx * sy * sz;
+        s.odd = odd[a];
+        int outer = 1;
+        if (a == 0) { s.ls = sx; s.es = 1; s.os = 0; s.nlines = (int)(sy * sz); }
+        else if (a == 1) { s.ls = 1; s.es = sx; s.os = sx * sy; s.nlines = (int)sx; outer = (int)sz; }
+        else { s.ls = 1; s.es = sx * sy; s.os = 0; s.nlines = (int)(sx * sy); }
+        with_width(fxg_width(p[a]->L, 1, 8, SMEM_CAP, 0), [&](auto w) {
+            constexpr int NL = decltype(w)::value;
+            const int m = fxg_groups(*p[a], 64 / NL, NL < 4 ? 48 : 192 / NL);
+            const size_t sm = 2 * (size_t)p[a]->L * (NL + (a == 0)) * sizeof(fxc);
+            const dim3 grid(cdiv(s.nlines, NL), outer, 6);
+            if (a == 0) {
+                smem_attr((const void*)kg_sym_fx<NL, true>, sm, FX_STATIC_SM);
+                kg_sym_fx<NL, true><<<grid, NL * m, sm, st>>>(*p[a], fx_tables(pl, a), s, buf);
+            } else {
+                smem_attr((const void*)kg_sym_fx<NL, false>, sm, FX_STATIC_SM);
+                kg_sym_fx<NL, false><<<grid, NL * m, sm, st>>>(*p[a], fx_tables(pl, a), s, buf);
+            }
+        });
+    }
+    if (nl) *nl += 3;
     return cudaGetLastError();
 }
 

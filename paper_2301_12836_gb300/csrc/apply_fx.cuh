@@ -178,16 +178,17 @@ __global__ void __launch_bounds__(LPB * FourStep<A LSM_COMMA B>::TPL, B == 32 ? 
 // z pass with the Green multiply
 // ---------------------------------------------------------------------------------------------
 
-// Fixed-point copy of the octant spectra g [6][NO]: gx [6][NO] = (G1, G0) of the real part, then of
-// the imaginary part, and ge [NO] = the point's exponent (fx.cuh).
-static __global__ void __launch_bounds__(NTH) k_fx_spectrum(const double2* __restrict__ g, long long NO, int4* __restrict__ gx,
-                                                     int* __restrict__ ge) {
+// The forms of the octant spectra, from their FP64 values times scale (1/P): gx [6][NO] = (G1, G0) of the
+// real part, then of the imaginary part, ge [NO] = the point's exponent (fx.cuh), g32 and gdf FP32 and
+// double-float copies (either may be null).  g and gx may be the same memory.
+static __global__ void __launch_bounds__(NTH) k_spectrum_forms(const double2* g, double scale, long long NO, int4* gx, int* __restrict__ ge,
+                                                               float2* __restrict__ g32, dfcplx* __restrict__ gdf) {
     for (long long i = (long long)blockIdx.x * NTH + threadIdx.x; i < NO; i += (long long)gridDim.x * NTH) {
         double2 v[6];
         unsigned mag = 0;
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
-            v[c] = g[c * NO + i];
+            v[c] = cscale(g[c * NO + i], scale);
             mag = max(mag, max(fx_mag(v[c].x), fx_mag(v[c].y)));
         }
         const FxScale sc(mag);
@@ -204,6 +205,8 @@ static __global__ void __launch_bounds__(NTH) k_fx_spectrum(const double2* __res
             w.w = (int)(fx_ll(q.y) - ((long long)w.z << 30));
             if (zero) w = make_int4(0, 0, 0, 0);
             gx[c * NO + i] = w;
+            if (g32) g32[c * NO + i] = make_float2((float)v[c].x, (float)v[c].y);
+            if (gdf) gdf[c * NO + i] = dfcplx{df_from(v[c].x), df_from(v[c].y)};
         }
     }
 }

@@ -305,4 +305,69 @@ __global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FftPlan 
     }
 }
 
+// ---- Green spectrum setup: FFT of lines that are even or odd about element 0 (and zero at L / 2),
+// stored as their first half 0 .. n, n = L / 2; outputs 0 .. n in place.  Component c of the six
+// (blockIdx.z) is odd when bit c of `odd` is set.  Line i of outer group o starts at o os + i ls, its
+// elements es apart; ROWS: es = 1, loads and stores run along the line.
+struct SymArgs {
+    long long cs, os, ls, es;
+    int nlines, odd;
+};
+template <int NL, bool ROWS>
+__global__ void __launch_bounds__(NL * 48) kg_sym_fx(FftPlan p, FxTables T, SymArgs a, double2* __restrict__ buf) {
+    constexpr int LD = ROWS ? NL + 1 : NL;
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ unsigned s_mag[NL];
+    const int n = p.L / 2, i0 = blockIdx.x * NL;
+    const int l = threadIdx.x % NL, g = threadIdx.x / NL, m = blockDim.x / NL;
+    const int live = a.nlines - i0 < NL ? a.nlines - i0 : NL;
+    double2* tile = buf + blockIdx.z * a.cs + blockIdx.y * a.os + i0 * a.ls;
+    fxc* sa = reinterpret_cast<fxc*>(smem_raw);
+    fxc* sb = sa + (size_t)p.L * LD;
+    double2* raw = reinterpret_cast<double2*>(sb);
+    if (threadIdx.x < NL) s_mag[threadIdx.x] = 0;
+    __syncthreads();
+    if constexpr (ROWS) {
+        for (int k = 0; k < live; ++k) {
+            unsigned mag = 0;
+            for (int e = threadIdx.x; e <= n; e += blockDim.x) {
+                const double2 v = tile[k * a.ls + e];
+                raw[e * LD + k] = v;
+                mag = max(mag, max(fx_mag(v.x), fx_mag(v.y)));
+            }
+            if (mag) atomicMax(&s_mag[k], mag);
+        }
+    } else {
+        const unsigned mag = fxg_load<LD>(raw, n + 1, l, g, m, [&](int e) { return l < live ? tile[l * a.ls + e * a.es] : czero<double2>(); });
+        atomicMax(&s_mag[l], mag);
+    }
+    __syncthreads();
+    const FxScale sc(s_mag[l]);
+    const bool odd = (a.odd >> blockIdx.z & 1) != 0;
+    if (l < live)
+        for (int e = g; e < p.L; e += m) {
+            fxc v = fx_from(raw[(e <= n ? e : p.L - e) * LD + l], sc, p.fxbits);
+            if (odd && e > n) v = fxc{fx_neg(v.x), fx_neg(v.y)};
+            sa[e * LD + l] = v;
+        }
+    __syncthreads();
+    const fxc* r = fxg_fft<-1, LD>(sa, sb, p, T, l, g, m);
+    if constexpr (ROWS) {
+        for (int k = 0; k < live; ++k) {
+            const FxScale sk(s_mag[k]);
+            const FxUnit un(sk.unit(p.fxbits) + p.fxsum, sk.bad, s_mag[k] == 0);
+            for (int e = threadIdx.x; e <= n; e += blockDim.x) {
+                const fxc v = r[e * LD + k];
+                tile[k * a.ls + e] = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
+            }
+        }
+    } else if (l < live) {
+        const FxUnit un(sc.unit(p.fxbits) + p.fxsum, sc.bad, s_mag[l] == 0);
+        for (int e = g; e <= n; e += m) {
+            const fxc v = r[e * LD + l];
+            tile[l * a.ls + e * a.es] = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
+        }
+    }
+}
+
 }  // namespace lsm

@@ -57,6 +57,12 @@ __device__ __forceinline__ dfloat df_split(double v, int e) {
     return dfloat(__uint_as_float(sign | hb), sign ? -lo : lo);
 }
 
+// v as a pair: hi = fl32(v), lo = fl32(v - hi)
+__device__ __forceinline__ dfloat df_from(double v) {
+    const float h = __double2float_rn(v);
+    return dfloat(h, __double2float_rn(v - (double)h));
+}
+
 // s + e = a + b exactly
 __device__ __forceinline__ dfloat df_two_sum(float a, float b) {
     const float s = __fadd_rn(a, b);

@@ -101,15 +101,19 @@ __device__ void radial(const GreenPar& p, double r, double ir, double2& f, doubl
     }
 }
 
-// Table on the 2n-periodic grid, [6][Lz][Ly][Lx], components (11, 22, 33, 23, 13, 12):
-// h^3 G(m h) for |m_a| <= n_a - 1, m != 0; self-cell value at m = 0; zero on planes m_a = n_a.
+// Kernel table h^3 G(m h), components (11, 22, 33, 23, 13, 12): self-cell value at m = 0, zero on the
+// planes m_a = n_a.  On the whole 2n-periodic grid [6][Lz][Ly][Lx] (m_a in -n_a .. n_a - 1), or only its
+// octant m_a = 0 .. n_a, [6][nz+1][ny+1][nx+1], of which the rest is the mirror image (G_ij is odd in
+// the axes i and j where i != j, even in the others).
+template <bool OCTANT>
 __global__ void k_green_table(Dims d, GreenPar p, double2 self, double2* __restrict__ T) {
-    const long long P = (long long)d.Lx * d.Ly * d.Lz;
+    const int sx = OCTANT ? d.nx + 1 : d.Lx, sy = OCTANT ? d.ny + 1 : d.Ly, sz = OCTANT ? d.nz + 1 : d.Lz;
+    const long long P = (long long)sx * sy * sz;
     const double h3 = d.h * d.h * d.h;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
-        const int ix = (int)(i % d.Lx);
-        const int iy = (int)((i / d.Lx) % d.Ly);
-        const int iz = (int)(i / ((long long)d.Lx * d.Ly));
+        const int ix = (int)(i % sx);
+        const int iy = (int)((i / sx) % sy);
+        const int iz = (int)(i / ((long long)sx * sy));
         double2 out[6];
         for (int c = 0; c < 6; ++c) out[c] = make_double2(0.0, 0.0);
         if (ix != d.nx && iy != d.ny && iz != d.nz) {
@@ -299,20 +303,37 @@ static inline int gsz(long long n) {
 cudaError_t fft3_inplace_setup(const Dims& d, const Plans& pl, double2* buf, int ncomp, cudaStream_t st, long long* nl);
 cudaError_t launch_extract_octant(const Dims& d, const double2* full, double2* oct, double scale, cudaStream_t st, long long* nl);
 
+// Cell average of G over [-h/2, h/2]^3 times h^3, to O(w h): the static Kelvin part gives
+// (1/(3a^2) + 2/(3b^2)) C h^2 / (4 pi rho) with C = int_{unit cube} dV/|x| = 3 ln(2+sqrt3) - pi/2,
+// the r^0 term of the expansion gives i w h^3 (1/(3a^3) + 2/(3b^3)) / (4 pi rho).
+static double2 self_cell(const GreenPar& p, double h) {
+    const double Cself = 3.0 * log(2.0 + sqrt(3.0)) - 0.5 * M_PI;
+    const double c4 = 1.0 / (4.0 * M_PI * p.rho);
+    double2 self;
+    self.x = c4 * (1.0 / (3.0 * p.a * p.a) + 2.0 / (3.0 * p.b * p.b)) * Cself * h * h;
+    self.y = c4 * p.w * (1.0 / (3.0 * p.a * p.a * p.a) + 2.0 / (3.0 * p.b * p.b * p.b)) * h * h * h;
+    return self;
+}
+
+cudaError_t launch_green_octant(const Dims& d, const Plans& pl64, double lam, double mu, double rho, double omega, int green,
+                                int4* gx, int* ge, float2* g32, dfcplx* gdf, cudaStream_t st, long long* nl) {
+    const GreenPar p = make_green_par(lam, mu, rho, omega, green);
+    const long long NO = (long long)(d.nx + 1) * (d.ny + 1) * (d.nz + 1);
+    double2* buf = reinterpret_cast<double2*>(gx);   // FP64 until the last kernel, which converts in place
+    k_green_table<true><<<gsz(NO), 256, 0, st>>>(d, p, self_cell(p, d.h), buf);
+    if (nl) *nl += 1;
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_octant_fft(d, pl64, buf, st, nl);
+    if (e == cudaSuccess) e = launch_spectrum_forms(buf, 1.0 / ((double)d.Lx * d.Ly * d.Lz), NO, gx, ge, g32, gdf, st, nl);
+    return e;
+}
+
 cudaError_t launch_green_setup(const Dims& d, const Plans& pl64, double lam, double mu, double rho, double omega,
                                int green, int kernel, double2* scratch, double2* ghat64, cudaStream_t st, long long* nl) {
     const GreenPar p = make_green_par(lam, mu, rho, omega, green);
-    // cell average of G over [-h/2, h/2]^3 times h^3, to O(w h): the static Kelvin part gives
-    // (1/(3a^2) + 2/(3b^2)) C h^2 / (4 pi rho) with C = int_{unit cube} dV/|x| = 3 ln(2+sqrt3) - pi/2,
-    // the r^0 term of the expansion gives i w h^3 (1/(3a^3) + 2/(3b^3)) / (4 pi rho).
-    const double Cself = 3.0 * log(2.0 + sqrt(3.0)) - 0.5 * M_PI;
-    const double c4 = 1.0 / (4.0 * M_PI * rho);
-    const double h = d.h;
-    double2 self;
-    self.x = c4 * (1.0 / (3.0 * p.a * p.a) + 2.0 / (3.0 * p.b * p.b)) * Cself * h * h;
-    self.y = c4 * omega * (1.0 / (3.0 * p.a * p.a * p.a) + 2.0 / (3.0 * p.b * p.b * p.b)) * h * h * h;
+    const double2 self = self_cell(p, d.h);
     const long long P = (long long)d.Lx * d.Ly * d.Lz;
-    k_green_table<<<gsz(P), 256, 0, st>>>(d, p, self, scratch);
+    k_green_table<false><<<gsz(P), 256, 0, st>>>(d, p, self, scratch);
     if (nl) *nl += 1;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -405,11 +426,8 @@ __global__ void k_f2d_c(const float2* __restrict__ in, double2* __restrict__ out
 
 // double -> double-float: hi = fl32(v), lo = fl32(v - hi); |lo| <= ulp(hi) / 2
 __global__ void k_d2df(const double* __restrict__ in, dfloat* __restrict__ out, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const double v = in[i];
-        const float h = __double2float_rn(v);
-        out[i] = dfloat(h, __double2float_rn(v - (double)h));
-    }
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = df_from(in[i]);
 }
 // double-float -> double in place (hi + lo rounded once to FP64)
 __global__ void k_df2d(double* buf, long long n) {

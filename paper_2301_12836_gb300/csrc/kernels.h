@@ -112,8 +112,15 @@ cudaError_t launch_time_traces(int nf, double df, int ntr, const double2* U, int
 cudaError_t launch_gather_receivers(const double2* u, long long N, const long long* node, int nrec, double2* out,
                                     cudaStream_t st);
 
-// Fixed-point copy of six FP64 octant spectra for the z pass: gx [6][NO], ge [NO] (apply_fx.cuh).
-cudaError_t launch_fx_spectrum(const double2* ghat64, long long NO, int4* gx, int* ge, cudaStream_t st, long long* nlaunch);
+// The same spectrum from the octant of the table alone (difference form): gx [6][NO] and ge [NO], the
+// fixed-point form of the FP64 z pass (apply_fx.cuh), and the FP32 and double-float copies g32, gdf
+// (null: not wanted).  Works in gx itself, no scratch.
+cudaError_t launch_green_octant(const Dims& d, const Plans& pl64, double lam, double mu, double rho, double omega, int green,
+                                int4* gx, int* ge, float2* g32, dfcplx* gdf, cudaStream_t st, long long* nlaunch);
+// its steps in apply.cu: the three symmetric FFTs in place, and the forms of FP64 spectra times scale
+cudaError_t launch_octant_fft(const Dims& d, const Plans& pl64, double2* buf, cudaStream_t st, long long* nlaunch);
+cudaError_t launch_spectrum_forms(const double2* g, double scale, long long NO, int4* gx, int* ge, float2* g32, dfcplx* gdf,
+                                  cudaStream_t st, long long* nlaunch);
 
 // Precision converters.  d2df: n reals to double-float pairs; df2d_inplace: n double-float pairs
 // to doubles in the same memory (8 bytes each).

@@ -116,9 +116,12 @@ struct lsm_ctx {
     Store* s = nullptr;
     double omega = 0;
     lsm_opts o;
+    // octant spectra.  Sampled-H form: 24 planes each, own allocations.  Difference form: six planes in
+    // spec: gx, ge (the FP64 z pass's fixed-point form, apply_fx.cuh), ghat32, ghatdf; no FP64 copy.
+    void* spec = nullptr;
+    int4* gx = nullptr;
+    int* ge = nullptr;
     double2* ghat64 = nullptr;
-    int4* gx = nullptr;       // fixed-point copy of the G spectra for the FP64 z pass, and ...
-    int* ge = nullptr;        // ... its exponent per point (in gx's allocation)
     float2* ghat32 = nullptr;
     dfcplx* ghatdf = nullptr;
     long long nl = 0;
@@ -327,8 +330,26 @@ static lsm_status build_spectrum(lsm_t h) {
     Store* s = h->s;
     const Dims& d = s->d;
     const long long NO = (long long)(d.nx + 1) * (d.ny + 1) * (d.nz + 1);
+    if (s->kernel == LSM_KERNEL_DIFF) {
+        // one allocation for the spectrum's forms: fixed point, its exponents, FP32, double-float
+        const size_t b0 = 6 * NO * sizeof(int4), b1 = (NO * sizeof(int) + 255) & ~(size_t)255;
+        const size_t b2 = s->precision == LSM_MIXED ? (6 * NO * sizeof(float2) + 255) & ~(size_t)255 : 0;
+        const size_t b3 = s->pair ? 6 * NO * sizeof(dfcplx) : 0;
+        const size_t o1 = (b0 + 255) & ~(size_t)255;
+        char* b = nullptr;
+        CK(h, cudaMalloc(&b, o1 + b1 + b2 + b3));
+        h->spec = b;
+        h->gx = (int4*)b;
+        h->ge = (int*)(b + o1);
+        if (b2) h->ghat32 = (float2*)(b + o1 + b1);
+        if (b3) h->ghatdf = (dfcplx*)(b + o1 + b1 + b2);
+        CK(h, launch_green_octant(d, s->pl64, s->lam, s->mu, s->rho, h->omega, s->green, h->gx, h->ge, h->ghat32, h->ghatdf, s->st,
+                                  &h->nl));
+        CK(h, cudaStreamSynchronize(s->st));
+        return LSM_OK;
+    }
     const long long P = (long long)d.Lx * d.Ly * d.Lz;
-    const long long planes = s->kernel == LSM_KERNEL_H ? 24 : 6;
+    const long long planes = 24;
     CK(h, cudaMalloc(&h->ghat64, planes * NO * sizeof(double2)));
     double2* scratch = nullptr;
     CK(h, cudaMalloc(&scratch, 6 * P * sizeof(double2)));
@@ -337,12 +358,6 @@ static lsm_status build_spectrum(lsm_t h) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
     cudaFree(scratch);
     if (e != cudaSuccess) return cuda_fail(h, e, "green spectrum setup");
-    if (s->kernel == LSM_KERNEL_DIFF) {
-        CK(h, cudaMalloc(&h->gx, 6 * NO * sizeof(int4) + NO * sizeof(int)));
-        h->ge = (int*)(h->gx + 6 * NO);
-        CK(h, launch_fx_spectrum(h->ghat64, NO, h->gx, h->ge, s->st, &h->nl));
-        CK(h, cudaStreamSynchronize(s->st));
-    }
     if (s->precision == LSM_MIXED) {
         CK(h, cudaMalloc(&h->ghat32, planes * NO * sizeof(float2)));
         CK(h, launch_d2f((const double*)h->ghat64, (float*)h->ghat32, 2 * planes * NO, s->st, &h->nl));
@@ -497,10 +512,13 @@ extern "C" lsm_status lsm_create_shared(lsm_t* out, lsm_t base, double omega) {
 
 extern "C" void lsm_destroy(lsm_t h) {
     if (!h) return;
-    cudaFree(h->ghat64);
-    cudaFree(h->gx);
-    cudaFree(h->ghat32);
-    cudaFree(h->ghatdf);
+    if (h->spec) {
+        cudaFree(h->spec);
+    } else {
+        cudaFree(h->ghat64);
+        cudaFree(h->ghat32);
+        cudaFree(h->ghatdf);
+    }
     store_release(h->s);
     delete h;
 }
