@@ -235,7 +235,8 @@ __global__ void k_source(Dims d, GreenPar p, MomentSet ms, double sx, double sy,
 
 // Re<lam, d u0/d M_J> for the unit Voigt moments e_J (M23 = M32 = 1 for J = 3, and so on):
 // u0_i(e_J) = -[(f' + g/r) (E_J g)_i + (g' - 2 g/r)(g.E_J g) g_i + (g/r) tr(E_J) g_i].
-// Block b writes its six partial sums to partial[b * 6 + J]; k_sum6 adds them in block order.
+// Block b writes its six partial sums to partial[b * 6 + J]; k_sum6 adds them in a fixed order.
+// FP64-bound; evaluated moment by moment the sums took as many operations again (96^3: 573 us).
 constexpr int SG_BLOCKS = 4096;
 __global__ void __launch_bounds__(256) k_source_grad(Dims d, GreenPar p, double sx, double sy, double sz,
                                                      const double2* __restrict__ lamv, double* __restrict__ partial) {
@@ -255,24 +256,22 @@ __global__ void __launch_bounds__(256) k_source_grad(Dims d, GreenPar p, double 
         const double2 A = make_double2(fp.x + gg.x * ir, fp.y + gg.y * ir);
         const double2 B = make_double2(gp.x - 2.0 * gg.x * ir, gp.y - 2.0 * gg.y * ir);
         const double2 Cc = make_double2(gg.x * ir, gg.y * ir);
-        double2 l[3];
-        for (int c = 0; c < 3; ++c) l[c] = lamv[c * N + i];
-        // Voigt pairs of e_J: 11, 22, 33, 23, 13, 12
-        const int pa[6] = {0, 1, 2, 1, 0, 0}, pb[6] = {0, 1, 2, 2, 2, 1};
-        for (int J = 0; J < 6; ++J) {
-            double Mg[3] = {0, 0, 0};
-            Mg[pa[J]] += g[pb[J]];
-            if (pa[J] != pb[J]) Mg[pb[J]] += g[pa[J]];
-            const double gMg = g[0] * Mg[0] + g[1] * Mg[1] + g[2] * Mg[2];
-            const double tr = J < 3 ? 1.0 : 0.0;
-            double s = 0.0;
-            for (int c = 0; c < 3; ++c) {
-                const double s1 = Mg[c], s2 = gMg * g[c], s3 = tr * g[c];
-                const double ux = -(A.x * s1 + B.x * s2 + Cc.x * s3), uy = -(A.y * s1 + B.y * s2 + Cc.y * s3);
-                s += l[c].x * ux + l[c].y * uy;   // Re(conj(lam) u0)
-            }
-            acc[J] += s;
+        // Re(conj(lam) . u0(e_J)) = -[a . E_J g + (B', g.E_J g) + (C', tr E_J)] with a_c = Re(conj(lam_c) A),
+        // B' = Re(conj(L) B), C' = Re(conj(L) C), L = sum_c g_c lam_c: the six moments share all of it
+        double a[3], Lx = 0.0, Ly = 0.0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double2 l = lamv[c * N + i];
+            a[c] = l.x * A.x + l.y * A.y;
+            Lx += g[c] * l.x;
+            Ly += g[c] * l.y;
         }
+        const double b = Lx * B.x + Ly * B.y, t = Lx * Cc.x + Ly * Cc.y;
+#pragma unroll
+        for (int J = 0; J < 3; ++J) acc[J] -= (a[J] + b * g[J]) * g[J] + t;
+        acc[3] -= a[1] * g[2] + (a[2] + 2.0 * b * g[2]) * g[1];
+        acc[4] -= a[0] * g[2] + (a[2] + 2.0 * b * g[2]) * g[0];
+        acc[5] -= a[0] * g[1] + (a[1] + 2.0 * b * g[1]) * g[0];
     }
     __shared__ double sh[6][256];
     for (int J = 0; J < 6; ++J) sh[J][threadIdx.x] = acc[J];
@@ -286,12 +285,15 @@ __global__ void __launch_bounds__(256) k_source_grad(Dims d, GreenPar p, double 
         for (int J = 0; J < 6; ++J) partial[blockIdx.x * 6 + J] = sh[J][0];
 }
 
+// out[J] = sum over blocks of partial[b * 6 + J]: one warp per J, lane sums in block order, then a
+// shuffle tree (one thread per J took 250 us for 3456 blocks)
 __global__ void k_sum6(const double* __restrict__ partial, int nblk, double* __restrict__ out) {
-    if (threadIdx.x < 6) {
-        double s = 0.0;
-        for (int b = 0; b < nblk; ++b) s += partial[b * 6 + threadIdx.x];
-        out[threadIdx.x] = s;
-    }
+    const int J = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int b = lane; b < nblk; b += 32) s += partial[b * 6 + J];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) out[J] = s;
 }
 
 static inline int gsz(long long n) {
@@ -380,7 +382,7 @@ cudaError_t launch_source_gradient(const Dims& d, double lam, double mu, double 
     if (nb > SG_BLOCKS) nb = SG_BLOCKS;
     if (nb < 1) nb = 1;
     k_source_grad<<<(int)nb, 256, 0, st>>>(d, p, xs[0], xs[1], xs[2], lamv, partial);
-    k_sum6<<<1, 32, 0, st>>>(partial, (int)nb, out);
+    k_sum6<<<1, 192, 0, st>>>(partial, (int)nb, out);
     if (nl) *nl += 2;
     return cudaGetLastError();
 }
