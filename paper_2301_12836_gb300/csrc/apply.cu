@@ -149,6 +149,10 @@ __device__ __forceinline__ void stress_at(const Dims& d, const T* __restrict__ d
     }
 }
 
+// Threads of a node kernel's block: a constant for the memory-bound types (as a variable it cost
+// k_stress<float>, held to 32 registers, 6% of an FP32 apply), the launch's choice in FP64
+template <typename T> __device__ __forceinline__ int node_dim() { return std::is_same<T, double>::value ? (int)blockDim.x : NTH; }
+
 template <typename T>
 __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? 8 : 2) k_stress(Dims d, const T* __restrict__ dC, const ApplySys<T>* __restrict__ sys) {
     typedef typename cplx_of<T>::type C;
@@ -158,7 +162,8 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? 8 : 2) k_stress(Dims d, 
     C* __restrict__ sig = S.w1;
     const long long N = d.N;
     const long long sxy = (long long)d.nx * d.ny;
-    for (long long idx = (long long)blockIdx.x * NTH + threadIdx.x; idx < N; idx += (long long)gridDim.x * NTH) {
+    const int nth = node_dim<T>();
+    for (long long idx = (long long)blockIdx.x * nth + threadIdx.x; idx < N; idx += (long long)gridDim.x * nth) {
         const int ix = (int)(idx % d.nx);
         const int iy = (int)((idx / d.nx) % d.ny);
         const int iz = (int)(idx / sxy);
@@ -738,7 +743,8 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? 6 : 1) k_divq(Dims d, co
     const long long E = (long long)d.ex * d.ey * d.ez;
     const long long sxy = (long long)d.nx * d.ny;
     const T i2h = (T)(0.5 / d.h);
-    for (long long idx = (long long)blockIdx.x * NTH + threadIdx.x; idx < E; idx += (long long)gridDim.x * NTH) {
+    const int nth = node_dim<T>();
+    for (long long idx = (long long)blockIdx.x * nth + threadIdx.x; idx < E; idx += (long long)gridDim.x * nth) {
         const int p0 = (int)(idx % d.ex) - 1;
         const int p1 = (int)((idx / d.ex) % d.ey) - 1;
         const int p2 = (int)(idx / ((long long)d.ex * d.ey)) - 1;
@@ -1119,7 +1125,8 @@ __global__ void __launch_bounds__(NTH) k_adj_stress(Dims d, const T* __restrict_
     const long long E = (long long)d.ex * d.ey * d.ez;
     const T i2h = (T)(0.5 / d.h);
     const long long sxy = (long long)d.nx * d.ny;
-    for (long long idx = (long long)blockIdx.x * NTH + threadIdx.x; idx < N; idx += (long long)gridDim.x * NTH) {
+    const int nth = node_dim<T>();
+    for (long long idx = (long long)blockIdx.x * nth + threadIdx.x; idx < N; idx += (long long)gridDim.x * nth) {
         const int ix = (int)(idx % d.nx);
         const int iy = (int)((idx / d.nx) % d.ny);
         const int iz = (int)(idx / sxy);
@@ -1184,7 +1191,8 @@ __global__ void __launch_bounds__(NTH) k_adj_out(Dims d, const T* __restrict__ d
     const long long E = (long long)d.ex * d.ey * d.ez;
     const T ih = (T)(1.0 / d.h), i2h = (T)(0.5 / d.h);
     const long long sxy = (long long)d.nx * d.ny;
-    for (long long idx = (long long)blockIdx.x * NTH + threadIdx.x; idx < N; idx += (long long)gridDim.x * NTH) {
+    const int nth = node_dim<T>();
+    for (long long idx = (long long)blockIdx.x * nth + threadIdx.x; idx < N; idx += (long long)gridDim.x * nth) {
         const int ix = (int)(idx % d.nx);
         const int iy = (int)((idx / d.nx) % d.ny);
         const int iz = (int)(idx / sxy);
@@ -1266,6 +1274,18 @@ static int generic_rows_nl(int L, int shrink = 0) {
 
 static inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 
+// Threads per block of the FP64 node kernels: 256, halved down to a warp while the grid would leave SMs
+// idle.  They are bound by the FP64 pipe of the SMs that run them: at 16^3 (4096 nodes, 16 blocks of
+// 256) one apply takes 55.3 us, with 128 blocks of 32 49.2 us.
+template <typename T> static inline int node_threads(long long n) {
+    int th = NTH;
+    while (std::is_same<T, double>::value && th > 32 && n < 152LL * th) th /= 2;
+    return th;
+}
+template <typename T> static inline int grid_nodes(long long n) {
+    const long long b = cdiv(n, node_threads<T>(n));
+    return (int)(b < 152 * 16 ? b : 152 * 16);
+}
 static inline int grid_elems(long long n) {
     long long b = (n + NTH - 1) / NTH;
     if (b > 152 * 16) b = 152 * 16;
@@ -1511,7 +1531,7 @@ static void launch_fftx_out(const Dims& d, const ApplySys<T>* sys, int nsys, con
 // Plain FFT of lines of length L along a strided axis: a.ncomp components per system, lines along
 // x (a.nlines of them), `outer` line groups (blockIdx.y) per component.
 template <typename T, int DIR>
-static void launch_strided(int L, const FftPlan& p, const void* tw, const Plans& pl, int axis, StridedArgs a, int outer,
+static void launch_strided(int L, const FxPlan& p, const void* tw, const Plans& pl, int axis, StridedArgs a, int outer,
                            const ApplySys<T>* sys, int nsys, cudaStream_t st, int v = 0) {
     typedef typename cplx_of<T>::type C;
     if (!fourstep_prunable(L, DIR < 0 ? a.in_off + a.in_count : 0, DIR > 0 ? a.out_off + a.out_count : 0)) v = 1;
@@ -1729,7 +1749,7 @@ static cudaError_t launch_apply_h(const Medium& m, const Plans& pl, const ApplyS
     const long long P = (long long)d.Lx * d.Ly * d.Lz;
     // 1. stress -> w1 planes 0..5, w^2 drho u -> planes 6..8 ([9][nz][ny][nx])
     ktimer_mark(tm, 0, f32, st, 0);
-    k_stress<T><<<dim3(grid_elems(d.N), nsys), NTH, 0, st>>>(d, (const T*)m.dC, sys);
+    k_stress<T><<<dim3(grid_nodes<T>(d.N), nsys), node_threads<T>(d.N), 0, st>>>(d, (const T*)m.dC, sys);
     k_hrho<T><<<dim3(grid_elems(d.N), nsys), NTH, 0, st>>>(d, (const T*)m.drho, sys);
     ktimer_mark(tm, 0, f32, st, 1);
     // 2. forward x FFT of the 9 planes: w1 -> w2 [9][nz][ny][Lx]
@@ -1790,11 +1810,12 @@ cudaError_t launch_apply(const Medium& m, const Plans& pl, const ApplySys<T>* sy
     } else {
         // 1. strain + contraction -> w1 [6][N]
         ktimer_mark(tm, 0, f32, st, 0);
-        k_stress<T><<<dim3(grid_elems(d.N), nsys), NTH, 0, st>>>(d, dC, sys);
+        k_stress<T><<<dim3(grid_nodes<T>(d.N), nsys), node_threads<T>(d.N), 0, st>>>(d, dC, sys);
         ktimer_mark(tm, 0, f32, st, 1);
         // 2. contrast source on the extended nodes -> w2 [3][ez][ey][ex]; forward x FFT -> w1 [3][ez][ey][Lx]
         ktimer_mark(tm, 1, f32, st, 0);
-        k_divq<T><<<dim3(grid_elems((long long)d.ex * d.ey * d.ez), nsys), NTH, 0, st>>>(d, drho, sys);
+        const long long E = (long long)d.ex * d.ey * d.ez;
+        k_divq<T><<<dim3(grid_nodes<T>(E), nsys), node_threads<T>(E), 0, st>>>(d, drho, sys);
         launch_xfwd<T>(d, sys, nsys, pl, st, sched[1]);
         ktimer_mark(tm, 1, f32, st, 1);
     }
@@ -1842,9 +1863,9 @@ cudaError_t launch_adjoint(const Medium& m, const Plans& pl, const ApplySys<T>* 
     const T* drho = (const T*)m.drho;
     launch_adjoint_conv<T>(m, pl, sys, nsys, st);
     // 6. transposed divergence + contraction -> w2 [6][N]
-    k_adj_stress<T><<<dim3(grid_elems(d.N), nsys), NTH, 0, st>>>(d, dC, sys);
+    k_adj_stress<T><<<dim3(grid_nodes<T>(d.N), nsys), node_threads<T>(d.N), 0, st>>>(d, dC, sys);
     // 7. transposed strain + density, AH w = w - (...)
-    k_adj_out<T><<<dim3(grid_elems(d.N), nsys), NTH, 0, st>>>(d, drho, sys);
+    k_adj_out<T><<<dim3(grid_nodes<T>(d.N), nsys), node_threads<T>(d.N), 0, st>>>(d, drho, sys);
     if (nl) *nl += 7;
     return cudaGetLastError();
 }
@@ -1877,7 +1898,7 @@ __global__ void __launch_bounds__(NTH) k_grad(Dims d, const ApplySys<double>* __
     const long long E = (long long)d.ex * d.ey * d.ez;
     const double ih = 1.0 / d.h, i2h = 0.5 / d.h;
     const long long sxy = (long long)d.nx * d.ny;
-    for (long long idx = (long long)blockIdx.x * NTH + threadIdx.x; idx < N; idx += (long long)gridDim.x * NTH) {
+    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += (long long)gridDim.x * blockDim.x) {
         const int ix = (int)(idx % d.nx);
         const int iy = (int)((idx / d.nx) % d.ny);
         const int iz = (int)(idx / sxy);
@@ -1933,7 +1954,7 @@ __global__ void __launch_bounds__(NTH) k_grad(Dims d, const ApplySys<double>* __
 cudaError_t launch_gradient(const Medium& m, const Plans& pl, const ApplySys<double>* sys, const double2* u, double* gC,
                             double* grho, int accumulate, cudaStream_t st, long long* nl) {
     launch_adjoint_conv<double>(m, pl, sys, 1, st);
-    k_grad<<<grid_elems(m.d.N), NTH, 0, st>>>(m.d, sys, u, gC, grho, accumulate);
+    k_grad<<<grid_nodes<double>(m.d.N), node_threads<double>(m.d.N), 0, st>>>(m.d, sys, u, gC, grho, accumulate);
     if (nl) *nl += 6;
     return cudaGetLastError();
 }
@@ -2009,8 +2030,8 @@ cudaError_t launch_octant_fft(const Dims& d, const Plans& pl, double2* buf, cuda
     const long long sx = d.nx + 1, sy = d.ny + 1, sz = d.nz + 1;
     // components odd along each axis (order 11, 22, 33, 23, 13, 12)
     const int odd[3] = {1 << 4 | 1 << 5, 1 << 3 | 1 << 5, 1 << 3 | 1 << 4};
-    const FftPlan* p[3] = {&pl.px, &pl.py, &pl.pz};
-    for (int a = 0; a < 3; ++a) {
+    const FxPlan* p[3] = {&pl.px, &pl.py, &pl.pz};
+    for (int a = 2; a >= 0; --a) {
         SymArgs s;
         s.cs = sx * sy * sz;
         s.odd = odd[a];

@@ -58,7 +58,7 @@ __device__ __forceinline__ void fxg_stage(const fxc* __restrict__ src, fxc* __re
 // Transform the tile in a (layout a[e * LD + l]); b is scratch of the same size.  Returns the buffer
 // of the result.  The caller synchronises before; the result is visible to the block on return.
 template <int S, int LD>
-__device__ __forceinline__ fxc* fxg_fft(fxc* a, fxc* b, const FftPlan& p, const FxTables& T, int l, int g, int m) {
+__device__ __forceinline__ fxc* fxg_fft(fxc* a, fxc* b, const FxPlan& p, const FxTables& T, int l, int g, int m) {
     int Ns = 1;
     for (int s = 0; s < p.nst; ++s) {
         const int R = p.radix[s];
@@ -77,7 +77,7 @@ __device__ __forceinline__ fxc* fxg_fft(fxc* a, fxc* b, const FftPlan& p, const 
 }
 
 // Groups per line, m <= most: the fewest butterfly rounds weighted by their size, then the most groups.
-static inline int fxg_groups(const FftPlan& p, int least, int most) {
+static inline int fxg_groups(const FxPlan& p, int least, int most) {
     int best = least;
     double cost = 1e300;
     for (int m = least; m <= most; ++m) {
@@ -116,7 +116,7 @@ __device__ __forceinline__ unsigned fxg_load(double2* raw, int n, int l, int g, 
 
 // ---- strided pass: NL consecutive lines along x per block
 template <int DIR, int NL>
-__global__ void __launch_bounds__(NL * 48) kg_strided_fx(FftPlan p, FxTables T, StridedArgs a, const ApplySys<double>* __restrict__ sys) {
+__global__ void __launch_bounds__(NL * 48) kg_strided_fx(FxPlan p, FxTables T, StridedArgs a, const ApplySys<double>* __restrict__ sys) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ unsigned s_mag[NL];
     const ApplySys<double>& S = sys[blockIdx.z / a.ncomp];
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(NL * 48) kg_strided_fx(FftPlan p, FxTables T, 
 // ---- contiguous rows: NL rows per block.  Row r of src holds in_count elements (placed at in_off),
 // row r of dst out_count (from out_off).  OUT: the inverse x pass's epilogue, dst = S.out = u - result.
 template <int DIR, int NL, bool OUT>
-__global__ void __launch_bounds__(NL * 48) kg_rows_fx(FftPlan p, FxTables T, const ApplySys<double>* __restrict__ sys, int src_sel,
+__global__ void __launch_bounds__(NL * 48) kg_rows_fx(FxPlan p, FxTables T, const ApplySys<double>* __restrict__ sys, int src_sel,
                                                       int dst_sel, long long nrows, int in_count, int in_off, int out_count,
                                                       int out_off) {
     constexpr int LD = NL + 1;
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(NL * 48) kg_rows_fx(FftPlan p, FxTables T, con
 
 // ---- z pass with the Green multiply: TX columns of one ky, as k4_fftz_green_fx
 template <bool CONJ, int TX>
-__global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FftPlan p, FxTables T, const ApplySys<double>* __restrict__ sys,
+__global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FxPlan p, FxTables T, const ApplySys<double>* __restrict__ sys,
                                                                 int nsys, int in_count, int in_off, int out_count, int out_off,
                                                                 int src_sel, int dst_sel) {
     constexpr int NL = 3 * TX;
@@ -308,13 +308,14 @@ __global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FftPlan 
 // ---- Green spectrum setup: FFT of lines that are even or odd about element 0 (and zero at L / 2),
 // stored as their first half 0 .. n, n = L / 2; outputs 0 .. n in place.  Component c of the six
 // (blockIdx.z) is odd when bit c of `odd` is set.  Line i of outer group o starts at o os + i ls, its
-// elements es apart; ROWS: es = 1, loads and stores run along the line.
+// elements es apart; ROWS: es = 1, loads and stores run along the line.  Outputs that vanish by
+// symmetry come out as exact zeros (fx_to_odd).
 struct SymArgs {
     long long cs, os, ls, es;
     int nlines, odd;
 };
 template <int NL, bool ROWS>
-__global__ void __launch_bounds__(NL * 48) kg_sym_fx(FftPlan p, FxTables T, SymArgs a, double2* __restrict__ buf) {
+__global__ void __launch_bounds__(NL * 48) kg_sym_fx(FxPlan p, FxTables T, SymArgs a, double2* __restrict__ buf) {
     constexpr int LD = ROWS ? NL + 1 : NL;
     extern __shared__ unsigned char smem_raw[];
     __shared__ unsigned s_mag[NL];
@@ -358,14 +359,14 @@ __global__ void __launch_bounds__(NL * 48) kg_sym_fx(FftPlan p, FxTables T, SymA
             const FxUnit un(sk.unit(p.fxbits) + p.fxsum, sk.bad, s_mag[k] == 0);
             for (int e = threadIdx.x; e <= n; e += blockDim.x) {
                 const fxc v = r[e * LD + k];
-                tile[k * a.ls + e] = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
+                tile[k * a.ls + e] = fx_to_odd(v, un);
             }
         }
     } else if (l < live) {
         const FxUnit un(sc.unit(p.fxbits) + p.fxsum, sc.bad, s_mag[l] == 0);
         for (int e = g; e <= n; e += m) {
             const fxc v = r[e * LD + l];
-            tile[l * a.ls + e * a.es] = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
+            tile[l * a.ls + e * a.es] = fx_to_odd(v, un);
         }
     }
 }

@@ -130,8 +130,11 @@ struct FftPlan {
     int L;
     int nst;
     int radix[12];
-    // fixed-point runs of the plan (apply_fxg.cuh): K of each stage, bits of the inputs, and the sum
-    // of the K by which the outputs' unit is coarser than the inputs'
+};
+// With its fixed-point runs (apply_fxg.cuh): K of each stage, bits of the inputs, and the sum of the K
+// by which the outputs' unit is coarser than the inputs'.  (The other engines' kernels take the plan
+// alone: with these fields in it they ran 2% slower.)
+struct FxPlan : FftPlan {
     int fxk[12];
     int fxbits, fxsum;
 };

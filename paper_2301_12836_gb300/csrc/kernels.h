@@ -52,7 +52,7 @@ struct Medium {
 };
 
 struct Plans {
-    FftPlan px, py, pz;
+    FxPlan px, py, pz;
     const void* twx;     // twiddle tables of T: exp(-2 pi i k / L)
     const void* twy;
     const void* twz;

@@ -149,7 +149,7 @@ lsm_status cuda_fail(lsm_t h, cudaError_t e, const char* where) {
 // Scaling of a plan's fixed-point stages: in log2 of the largest modulus, the first stage's outputs and
 // every later stage's stay below 61.9 with the smallest K in 1 .. 3 that does it (K = 1 doubles the
 // values before a product, which needs them below 60.9).
-void fixed_point_scaling(FftPlan& p) {
+void fixed_point_scaling(FxPlan& p) {
     const double top = 61.9;
     const double g0 = log2((double)p.radix[0]);
     p.fxbits = (int)floor(top - 0.5 - g0);
@@ -165,7 +165,7 @@ void fixed_point_scaling(FftPlan& p) {
     }
 }
 
-bool factor_plan(int L, FftPlan& p) {
+bool factor_plan(int L, FxPlan& p) {
     p.L = L;
     p.nst = 0;
     int m = L;
@@ -212,7 +212,7 @@ void twiddle_table(int L, std::vector<double2>& t64, std::vector<float2>& t32, s
 
 bool lsm_grid_ok(int n) {
     if (n < 2 || 2 * n > 512) return false;
-    FftPlan p;
+    FxPlan p;
     return factor_plan(2 * n, p);
 }
 
