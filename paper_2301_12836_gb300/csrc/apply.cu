@@ -626,6 +626,168 @@ __global__ void __launch_bounds__(2 * TX * A, 3) k4z_pair(
     }
 }
 
+// Register-resident FP32 z pass for L = A * B, B = 2 A (32, 128, 512), two y rows per block as
+// k4z_pair.  A line has B threads: (qq, h), qq < A, h = 0, 1, in lanes NL apart.  Forward: step 1, one
+// A-point DFT per thread (t = h A + qq); after the exchange the B-point DFT of k1 = qq is an A-point DFT
+// of the even t by h = 0 and one of the odd t by h = 1, combined by one radix-2 layer over shuffles,
+// which leaves X[qq + A k2] for k2 = j + h A / 2 and k2 + A (j < A / 2) in the thread's A registers per
+// component.  The Green multiply runs there; the inverse takes the same factors backwards (radix-2
+// layer over shuffles, A-point DFTs giving n1 = 2 m + h, exchange, one A-point DFT per n1).  The
+// shared-memory kernel k4_fftz_green makes three exchanges per transform where this makes one and
+// shuffles half a line.  256^3 (L = 512), one system: 4.72 -> 2.73 ms; 64^3 (L = 128): 47 -> 43 us.
+template <bool CONJ, int A, int TX>
+__global__ void __launch_bounds__(4 * TX * A, A == 16 ? 2 : 4) k4z_pair2(
+    Dims d, const float2* __restrict__ tw, const ApplySys<float>* __restrict__ sys, int nsys, int in_count, int in_off,
+    int out_count, int out_off, int src_sel, int dst_sel) {
+    typedef float2 C;
+    constexpr int B = 2 * A, L = A * B, NL = 2 * TX, NT = NL * B, NZ = A / 2 + 1, HA = A / 2;
+    constexpr int E = 16;
+    constexpr int YS = A * NL + (((NL - A * NL) % E) + E) % E;   // row stride of Y[t][.]
+    static_assert(NL <= 16, "the two halves of a line share a warp");
+    const int nin = in_off + in_count;
+    extern __shared__ unsigned char smem_raw[];
+    C* sY = reinterpret_cast<C*>(smem_raw);   // exchange buffer [B][YS]
+    C* sG = sY + B * YS;                      // [6][nz+1][TX] spectrum slice
+    C* sW = sG + 6 * (d.nz + 1) * TX;         // twiddles exp(-2 pi i k / L), k < L
+    const int lx = threadIdx.x % TX;
+    const int r = (threadIdx.x / TX) & 1;
+    const int l = lx + TX * r;
+    const int h = (threadIdx.x / NL) & 1;
+    const int q0 = threadIdx.x / (2 * NL);
+    const int j = blockIdx.y;                 // 0 .. ny
+    const bool alone = j == 0 || j == d.ny;
+    const int ky = (r == 0 || alone) ? j : d.Ly - j;
+    const bool owner = r == 0 || !alone;
+    const int x0 = blockIdx.x * TX;
+    const int kx = x0 + lx;
+    const bool xin = kx < d.Lx;
+    const unsigned my = ky > d.ny ? SIGN_BIT : 0u;
+    const unsigned mx = kx > d.nx ? SIGN_BIT : 0u;
+    const long long NO = (long long)(d.nx + 1) * (d.ny + 1) * (d.nz + 1);
+    const int GC = (d.nz + 1) * TX;
+    const int plane = d.Ly * d.Lx;
+    const long long colofs = (long long)ky * d.Lx + kx;
+    for (int i = threadIdx.x; i < L; i += NT) sW[i] = tw[i];   // ordered before use by the first barrier
+    const C* staged = nullptr;
+    for (int si = 0; si < nsys; ++si) {
+        int q;   // through an opaque move, as in k4z_pair: recomputed per system, not held across systems
+        asm volatile("mov.u32 %0, %1;" : "=r"(q) : "r"(q0));
+        const ApplySys<float> S = sys[si];
+        if (S.run && !*S.run) continue;
+        const bool fresh = S.ghat != staged;
+        if (fresh) {
+            __syncthreads();
+            const int lxx = threadIdx.x % TX;
+            const int kxx = x0 + lxx;
+            const int fx = kxx <= d.nx ? kxx : d.Lx - kxx;
+            int row = threadIdx.x / TX;
+            for (int i = threadIdx.x; i < 6 * GC; i += NT, row += NT / TX) {
+                const int c = row / (d.nz + 1);
+                const int fz = row - c * (d.nz + 1);
+                if (kxx < d.Lx)
+                    cp_async_elem(&sG[i], S.ghat + c * NO + ((long long)fz * (d.ny + 1) + j) * (d.nx + 1) + fx);
+            }
+            cp_async_commit();
+            staged = S.ghat;
+        }
+        const int t = h * A + q;
+        const C* __restrict__ src = pick<C>(S, src_sel) + colofs;
+        C R[3][A];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            C v[A];
+            const C* xc = src + (long long)c * in_count * plane;
+#pragma unroll
+            for (int a = 0; a < A; ++a) {
+                const int e = t + B * a;
+                const int es = e - in_off;
+                v[a] = (a < NZ && e < nin && es >= 0 && xin) ? xc[(long long)es * plane] : czero<C>();
+            }
+            dft_reg_p<A, -1, NZ, A>(v);
+            if (t) {
+#pragma unroll
+                for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], lds_fresh(&sW[t * k1]));
+            }
+            __syncthreads();   // the buffer's last reads are done (and the twiddle fill)
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) sY[t * YS + k1 * NL + l] = v[k1];
+            __syncthreads();
+#pragma unroll
+            for (int m = 0; m < A; ++m) R[c][m] = sY[(2 * m + h) * YS + q * NL + l];
+            dft_reg<A, -1>(R[c]);
+            if (h) {
+#pragma unroll
+                for (int k = 1; k < A; ++k) R[c][k] = cmul(R[c][k], lds_fresh(&sW[k * A]));   // W_B^k
+            }
+#pragma unroll
+            for (int k = 0; k < HA; ++k) {
+                const C s = h ? R[c][k] : R[c][k + HA];
+                C o;
+                o.x = __shfl_xor_sync(0xffffffffu, s.x, NL);
+                o.y = __shfl_xor_sync(0xffffffffu, s.y, NL);
+                const C e = h ? o : R[c][k], w = h ? R[c][k + HA] : o;   // E and W O of k2 = k + h HA
+                R[c][k] = cadd(e, w);
+                R[c][k + HA] = csub(e, w);
+            }
+        }
+        if (fresh) {
+            cp_async_wait_all();
+            __syncthreads();
+        }
+        // ---- Green multiply: R[.][k] is k2 = k + h HA, R[.][k + HA] is A more
+        if (xin) {
+#pragma unroll
+            for (int k = 0; k < A; ++k) {
+                const int k2 = (k < HA ? k : k - HA + A) + h * HA;
+                const int kz = q + A * k2;
+                const int fz = kz <= d.nz ? kz : L - kz;
+                const unsigned mz = kz > d.nz ? SIGN_BIT : 0u;
+                const C* g = sG + fz * TX + lx;
+                const C G0 = g[0], G1 = g[GC], G2 = g[2 * GC];
+                const C G3 = flip_sign(g[3 * GC], my ^ mz);
+                const C G4 = flip_sign(g[4 * GC], mx ^ mz);
+                const C G5 = flip_sign(g[5 * GC], mx ^ my);
+                const C qa = R[0][k], qb = R[1][k], qc = R[2][k];
+                R[0][k] = gdot3<CONJ>(G0, qa, G5, qb, G4, qc);
+                R[1][k] = gdot3<CONJ>(G5, qa, G1, qb, G3, qc);
+                R[2][k] = gdot3<CONJ>(G4, qa, G3, qb, G2, qc);
+            }
+        }
+        C* __restrict__ dst = pick<C>(S, dst_sel) + colofs;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int k = 0; k < HA; ++k) {
+                const C s = cadd(R[c][k], R[c][k + HA]);
+                const C f = cmulc(csub(R[c][k], R[c][k + HA]), lds_fresh(&sW[(k + h * HA) * A]));
+                const C give = h ? s : f;
+                C o;
+                o.x = __shfl_xor_sync(0xffffffffu, give.x, NL);
+                o.y = __shfl_xor_sync(0xffffffffu, give.y, NL);
+                R[c][k] = h ? o : s;        // h = 0 collects the sums, h = 1 the differences
+                R[c][k + HA] = h ? f : o;
+            }
+            dft_reg<A, 1>(R[c]);            // R[c][m] belongs to n1 = 2 m + h
+#pragma unroll
+            for (int m = 0; m < A; ++m) R[c][m] = cmulc(R[c][m], lds_fresh(&sW[q * (2 * m + h)]));
+            __syncthreads();
+#pragma unroll
+            for (int m = 0; m < A; ++m) sY[(2 * m + h) * YS + q * NL + l] = R[c][m];
+            __syncthreads();
+            C v[A];
+#pragma unroll
+            for (int k = 0; k < A; ++k) v[k] = sY[t * YS + k * NL + l];
+            dft_reg_p<A, 1, A, NZ>(v);      // outputs n = t + B n2, n2 < A/2 + 1 only (checked at launch)
+            C* dc = dst + (long long)c * out_count * plane;
+#pragma unroll
+            for (int n2 = 0; n2 < NZ; ++n2) {
+                const int eo = t + B * n2 - out_off;
+                if (owner && xin && eo >= 0 && eo < out_count) dc[(long long)eo * plane] = v[n2];
+            }
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------------------------
 // z pass with the Green multiply: forward z FFT, u-hat = G-hat q-hat (conj G-hat for the
 // adjoint), inverse z FFT.  CTA: TX lines along x at one ky, all three components.
@@ -1598,7 +1760,7 @@ static void launch_zplain(const Dims& d, const ApplySys<T>* sys, int nsys, const
     launch_strided<T, DIR>(d.Lz, pl.pz, pl.twz, pl, 2, a, d.Ly, sys, nsys, st);
 }
 
-// schedule variant v: 0 default (register-resident kernel for FP32 and L = A * A), 1 / 2 generic
+// schedule variant v: 0 default (register-resident kernels for FP32, L = A * A and 2 A * A), 1 / 2 generic
 // engine (default / half tile), 3 the shared-memory four-step kernel for every precision
 template <typename T, bool CONJ>
 static void launch_zpass(const Dims& d, const ApplySys<T>* sys, int nsys, const Plans& pl, int in_count, int in_off,
@@ -1634,6 +1796,18 @@ static void launch_zpass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
             const int E = (int)(128 / sizeof(C));
             const int GS = 6 * TX + (((TX - 6 * TX) % E) + E) % E;
             sm += (size_t)(d.nz + 1) * GS * sizeof(C);  // spectrum slice
+        }
+        if constexpr (F::INPLACE && sizeof(T) == 4 && F::B_ == 2 * F::A_) {
+          if (v != 3 && in_off + in_count <= (F::A_ / 2 + 1) * F::B_ && out_off + out_count <= (F::A_ / 2 + 1) * F::B_) {
+            constexpr int A = F::A_, TXR = 4, NL = 2 * TXR, E = 16;
+            constexpr int YS = A * NL + (((NL - A * NL) % E) + E) % E;
+            const size_t smr = ((size_t)2 * A * YS + (size_t)6 * (d.nz + 1) * TXR + (size_t)2 * A * A) * sizeof(C);
+            smem_attr((const void*)k4z_pair2<CONJ, A, TXR>, smr);
+            k4z_pair2<CONJ, A, TXR><<<dim3(cdiv(d.Lx, TXR), d.ny + 1, 1), 4 * TXR * A, smr, st>>>(
+                d, (const float2*)pl.twz, (const ApplySys<float>*)sys, nsys, in_count, in_off, out_count, out_off,
+                src_sel, dst_sel);
+            return;
+          }
         }
         if constexpr (F::INPLACE && sizeof(T) == 4 && F::A_ == F::B_) {
           if (v != 3) {
