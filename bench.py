@@ -464,9 +464,11 @@ def fused_epilogue(n, precision, kernel, schedule):
 
 
 def stage_records(lsm, st_ms, st_launch, a64, a32, ms, n, kernel, pair, share, fused=False):
-    """Per-stage rooflines: FP32 stages against HBM (algorithmic bytes), FP64 stages against the
-    FP64 pipe (model flops); double-float stages (FP32 pipe) against the HBM floor of their bytes
-    with their FP64-equivalent rate.  fused: see fused_epilogue."""
+    """Per-stage rooflines: FP32 stages against HBM (algorithmic bytes); FP64 stages too, except the
+    stress, which is bound by the FP64 pipe (model flops): the transform stages run on the integer
+    pipes in fixed point, so their model flops per second (fp64_equivalent_tflops) may exceed that
+    pipe's peak; double-float stages (FP32 pipe) against the HBM floor of their bytes.  fused: see
+    fused_epilogue."""
     peak, _ = peaks()
     stages = []
     for slot in range(12):
@@ -496,7 +498,7 @@ def stage_records(lsm, st_ms, st_launch, a64, a32, ms, n, kernel, pair, share, f
                         "unit": "GB/s", "frac": round(gbs / peak, 4), "algorithmic_bytes_per_system_apply": round(nbytes),
                         "fp64_equivalent_tflops": round(fl * napp / (st_ms[slot] / 1e3) / 1e12, 4),
                         "model_flops_per_system_apply": fl})
-        else:
+        elif stage == 0:
             fl = sf(stage, n)
             ach = fl * napp / (st_ms[slot] / 1e3) / 1e12
             nbytes = sb(stage, n, 16, 8, share)
@@ -505,6 +507,14 @@ def stage_records(lsm, st_ms, st_launch, a64, a32, ms, n, kernel, pair, share, f
                         "model_flops_per_system_apply": fl,
                         "hbm_gbs": round(nbytes * napp / (st_ms[slot] / 1e3) / 1e9, 1),
                         "algorithmic_bytes_per_system_apply": round(nbytes)})
+        else:
+            fl = sf(stage, n)
+            nbytes = sb(stage, n, 16, 8, share)
+            gbs = nbytes * napp / (st_ms[slot] / 1e3) / 1e9
+            rec.update({"bound": "alu (integer pipes, fixed point)", "achieved": round(gbs, 1), "peak": peak,
+                        "unit": "GB/s", "frac": round(gbs / peak, 4), "algorithmic_bytes_per_system_apply": round(nbytes),
+                        "fp64_equivalent_tflops": round(fl * napp / (st_ms[slot] / 1e3) / 1e12, 4),
+                        "model_flops_per_system_apply": fl})
         if kernel == "diff":
             t = traffic_from_profile(stage, "mixed" if f32 else ("dfloat" if pair else "fp64"), n, share)
             if t is not None:

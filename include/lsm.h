@@ -96,8 +96,9 @@ typedef struct {
                           LSM_RESIDUAL_FP64 (default): FP64.  LSM_RESIDUAL_DFLOAT: double-float
                           pairs (two FP32 words, about 48 significand bits, unit roundoff near
                           2^-48; see lsm_apply_df) on the FP32 pipe, with the iterate scaled by a
-                          power of two to RMS(b) ~ 1 first: several times faster on this GPU,
-                          whose FP64 rate is 1/64 of its FP32 rate, but narrower than FP64.
+                          power of two to RMS(b) ~ 1 first: narrower than FP64 and about as fast
+                          (one 128^3 apply 2.3 ms, the FP64 apply, whose transforms run in 64-bit
+                          fixed point, 2.1 ms).
                           Adjoint solves always use FP64.  Ignored for LSM_FP64 handles. */
     int fused_dots;    /* LSM_MIXED, 1 (default): the inner products of an FP32 BiCGSTAB
                           iteration (<r^, v> for alpha, <t, s> and <t, t> for omega) are summed in

@@ -10,7 +10,8 @@
 //   k(4)_strided  inverse FFT along y, crop
 //   k(4)_fftx_out inverse FFT along x, crop, Au = u - u_s
 // Power-of-two line lengths 16..512 use the compile-time four-step FFT kernels (k4_*), any other
-// length the runtime mixed-radix Stockham kernels.
+// length the runtime mixed-radix Stockham kernels.  FP64 transforms run in 64-bit fixed point (fx.cuh):
+// k4_*_fx in apply_fx.cuh, kg_*_fx for the other lengths in apply_fxg.cuh.
 // Only three displacement-like components pass through the FFTs: the derivative of the
 // Green tensor in Eq. 8 is applied as the central difference D_k in real space, which is
 // exactly the factor i sin(k h)/h of the spectral form.  The contrast source q is shifted by
@@ -104,7 +105,7 @@ __device__ __forceinline__ void ghat_at(const C* __restrict__ g, const Dims& d, 
 // to the node itself at the ends, where the step is h instead of 2h, so all loads issue together;
 // FP32 (memory-bound) measured faster with the ends as branches.  Same arithmetic either way.
 // FP64 runs 2 blocks of 256 threads per SM (124 registers): 458 -> 406 us per system apply at
-// 128^3 against 1 block (149 registers).
+// 128^3 against 1 block (149 registers).  It is the one FP64 stage still bound by the FP64 pipe.
 template <typename T>
 __device__ __forceinline__ void stress_at(const Dims& d, const T* __restrict__ dC, const typename cplx_of<T>::type* __restrict__ u,
                                           long long idx, int ix, int iy, int iz, typename cplx_of<T>::type (&sg)[6]) {
@@ -1039,11 +1040,9 @@ __global__ void __launch_bounds__(LPB * A, sizeof(T) == 4 ? 4 : 1) k4_rows_w(con
     }
 }
 
-// blocks per SM each precision is compiled for: FP32 (with or without DOTS) fits 80 registers
-// for 3 blocks of 256 threads; FP64 and double-float keep the occupancy they reach unconstrained
-// (5 and 4 blocks of 128 threads at A = 16)
-template <typename T>
-constexpr int xout_min_blocks() { return sizeof(T) == 4 ? 3 : (std::is_same<T, dfloat>::value ? 4 : 5); }
+// blocks per SM each type is compiled for: FP32 (with or without DOTS) fits 80 registers for 3 blocks
+// of 256 threads; double-float keeps the occupancy it reaches unconstrained (4 blocks of 128 threads)
+template <typename T> constexpr int xout_min_blocks() { return sizeof(T) == 4 ? 3 : 4; }
 
 // inverse x FFT of the rows of w2 [3][nz][ny][L], crop to x = k - xoff in [0, nx) (at most
 // (A/2 + 1) A outputs), Au = u - u_s.
@@ -1614,7 +1613,7 @@ static void launch_xrows(const Dims& d, const ApplySys<T>* sys, int nsys, const 
             k4_rows_w<T, A, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * A, 0, st>>>((const C*)pl.twx, sys, src_sel, dst_sel,
                                                                                    nrows, in_count);
         } else if constexpr (F::INPLACE) {
-            constexpr int A = F::A_, B = F::B_, NL = 8 + (sizeof(T) == 4 ? 0 : 4);
+            constexpr int A = F::A_, B = F::B_, NL = 8;   // FP32 only: double-float has no A != B engine
             const size_t sm = (size_t)A * B * (NL + 1) * sizeof(C);
             smem_attr((const void*)k4_rows<T, -1, A, B, NL>, sm);
             k4_rows<T, -1, A, B, NL><<<dim3(cdiv(nrows, NL), nsys), NL * F::TPL, sm, st>>>(

@@ -943,8 +943,8 @@ static lsm_status solve_batched(int nsys, const lsm_t* hs_in, const void* const*
             a.u = V[i].x; a.out = V[i].v; a.run = nullptr; sx[i] = a;
             a.u = V[i].x; a.out = k[6]; a.run = nullptr; a64[i] = a;   // true residual at exit
         }
-        // FP64 iterations keep the vector kernels: the FP64 epilogue is bound by the FP64 pipe,
-        // so the same FP64 products cost it as much as a separate kernel that streams the vectors
+        // FP64 iterations keep the vector kernels: on the FP64 pipe the same products would cost
+        // the epilogue as much as a separate kernel that streams the vectors
         const bool fuse = false;
         CK(h0, cudaMemcpyAsync(w.vecs, V.data(), nsys * sizeof(V[0]), cudaMemcpyHostToDevice, st));
         CK(h0, cudaMemcpyAsync(w.sys_v, sv.data(), nsys * sizeof(sv[0]), cudaMemcpyHostToDevice, st));
