@@ -105,7 +105,7 @@ __device__ __forceinline__ void ghat_at(const C* __restrict__ g, const Dims& d, 
 // to the node itself at the ends, where the step is h instead of 2h, so all loads issue together;
 // FP32 (memory-bound) measured faster with the ends as branches.  Same arithmetic either way.
 // FP64 runs 2 blocks of 256 threads per SM (124 registers): 458 -> 406 us per system apply at
-// 128^3 against 1 block (149 registers).  It is the one FP64 stage still bound by the FP64 pipe.
+// 128^3 against 1 block (149 registers).  It and the divergence are what the FP64 pipe still bounds.
 template <typename T>
 __device__ __forceinline__ void stress_at(const Dims& d, const T* __restrict__ dC, const typename cplx_of<T>::type* __restrict__ u,
                                           long long idx, int ix, int iy, int iz, typename cplx_of<T>::type (&sg)[6]) {

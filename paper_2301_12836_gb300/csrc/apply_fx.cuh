@@ -15,7 +15,8 @@ template <int A, int B> struct FxStep {
 };
 
 // Strided pass: TX consecutive lines along x per block, as k4_strided.  bits: fx_bits of the line's
-// nonzero inputs.
+// nonzero inputs.  Bound by the integer-add pipe.  128^3, one system: 1.05 ms on the FP64 pipe, 0.175
+// here (0.6 GB at 3.5 TB/s).
 template <int DIR, int A, int B, int TX>
 __global__ void __launch_bounds__(TX * FourStep<A LSM_COMMA B>::TPL, B == 32 ? 2 : 4) k4_strided_fx(
     const int4* __restrict__ tw, StridedArgs a, const ApplySys<double>* __restrict__ sys, int bits) {
@@ -69,7 +70,9 @@ __global__ void __launch_bounds__(TX * FourStep<A LSM_COMMA B>::TPL, B == 32 ? 2
 
 // Contiguous rows: each line on TPL consecutive lanes of one warp, as k4_rows_w, for every A and B.
 // The line's exponent is a shuffle reduction over its lanes and the exchange between the steps a
-// tile of its own ordered by __syncwarp, so a block has no barrier.
+// tile of its own ordered by __syncwarp, so a block has no barrier.  Bound by the integer-add pipe.
+// 128^3, one system: inverse x pass 0.57 -> 0.124 ms, contrast source and forward x 0.76 -> 0.31 (of
+// which the source, on the FP64 pipe, 0.23).
 template <int DIR, int A, int B, int NZ, int NO, class Tw, class St>
 __device__ __forceinline__ void fx_row(double2 (&in)[FourStep<A, B>::I1][NZ], fxc* tl, const Tw* __restrict__ tw, int q, int bits, St st) {
     typedef FourStep<A, B> F;
@@ -270,10 +273,11 @@ template <int TX, int NT, typename V> __device__ __forceinline__ V column_max(V 
 // line l = c TX + lx at s[k NL + l].  The column's three lines share one exponent.  The multiply
 // leaves each point's products in their own exponent (the point's spectrum exponent, kept in sE);
 // the column's largest sets the inverse transform's, and the shift happens as its first step loads
-// them.  Small blocks (96 threads, 30 KB at L = 256) keep five of them resident, whose loads, barriers
-// and arithmetic overlap; the spectrum is read through the caches, where the other systems and the
-// mirrored rows find it again.  (One block for all systems in turn, hoisting what they share, spilled
-// 110 registers.)
+// them.  TX = 4: 192 threads at L = 256, two blocks per SM whose loads, barriers and arithmetic overlap
+// (TX = 2 with four to six smaller blocks: the same at 128^3, slower at 64^3 and 256^3); the spectrum is
+// read through the caches, where the other systems and the mirrored rows find it again.  (One block for
+// all systems in turn, hoisting what they share, spilled 110 registers.)  Bound by the wide multiplies'
+// pipe and its latencies.  128^3, one system: 5.21 ms on the FP64 pipe, 0.93 here.
 template <bool CONJ, int A, int B, int TX>
 __global__ void __launch_bounds__(3 * TX * FourStep<A LSM_COMMA B>::TPL, 2) k4_fftz_green_fx(
     Dims d, const int4* __restrict__ tw, const ApplySys<double>* __restrict__ sys, int nsys, int in_count, int in_off,
