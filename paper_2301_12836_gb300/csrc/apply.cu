@@ -948,54 +948,14 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? 6 : 1) k_divq(Dims d, co
     }
 }
 
-// four-step contiguous-rows FFT: NL rows per block, compile-time sizes, loads batched in registers.
-// Row r of src starts at src + r * in_count (placed at in_off), row r of dst at dst + r * out_count.
-template <typename T, int DIR, int A, int B, int NL>
-__global__ void __launch_bounds__(NL * FourStep<A LSM_COMMA B>::TPL, sizeof(T) == 8 ? 3 : 2) k4_rows(const typename cplx_of<T>::type* __restrict__ tw,
-                                                                  const ApplySys<T>* __restrict__ sys, int src_sel, int dst_sel,
-                                                                  long long nrows, int in_count, int in_off, int out_count,
-                                                                  int out_off) {
-    typedef typename cplx_of<T>::type C;
-    constexpr int L = A * B, TPL = FourStep<A, B>::TPL, NTHR = NL * TPL, LD = NL + 1, PER = L / TPL;
-    extern __shared__ unsigned char smem_raw[];
-    const ApplySys<T> S = sys[blockIdx.y];
-    if (S.run && !*S.run) return;
-    C* s = reinterpret_cast<C*>(smem_raw);
-    const C* __restrict__ src = pick<C>(S, src_sel);
-    C* __restrict__ dst = pick<C>(S, dst_sel);
-    const long long r0 = (long long)blockIdx.x * NL;
-    const int tid = threadIdx.x;
-    C v[PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int i = tid + k * NTHR;
-        const int e = i % L, l = i / L;
-        const long long row = r0 + l;
-        const int es = e - in_off;
-        v[k] = (row < nrows && es >= 0 && es < in_count) ? src[row * in_count + es] : czero<C>();
-    }
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int i = tid + k * NTHR;
-        s[(i % L) * LD + i / L] = v[k];
-    }
-    __syncthreads();
-    fft4_smem<A, B, DIR, (DIR < 0 ? A / 2 + 1 : A), (DIR > 0 ? B / 2 + 1 : B)>(s, NL, LD, tw, tid);   // as in k4_strided
-    for (int i = tid; i < NL * out_count; i += NTHR) {
-        const int e = i % out_count, l = i / out_count;
-        const long long row = r0 + l;
-        if (row < nrows) dst[row * out_count + e] = s[(e + out_off) * LD + l];
-    }
-}
-
 // Two-step FFT of contiguous rows for L = A * A with each line held by A consecutive lanes of one
 // warp: lane q owns the step-1 DFT of t = q and the step-2 DFT of k1 = q.  Step 1 loads its inputs
 // x[t + A a] straight from global memory (for each a the line's lanes read A consecutive
 // elements), the transpose between the steps goes through a shared-memory tile private to the
 // line (row stride A + 1: conflict-free both ways) ordered by __syncwarp, and step 2 leaves
 // X[k1 + A k2] in registers for a coalesced store.  No block barrier and one shared-memory round
-// trip per element (the tile-transposing kernels above make three).  The arithmetic is that of
-// fft4_smem, operation for operation, so results are bitwise those of k4_rows / k4_fftx_out.
+// trip per element (a tile-transposing kernel makes three).  The arithmetic is that of fft4_smem,
+// operation for operation.
 template <int A, typename C>
 __device__ __forceinline__ void rows_w_exchange(C (&v)[A], C* tl, int q) {
 #pragma unroll
@@ -1158,64 +1118,98 @@ __global__ void __launch_bounds__(LPB * A, xout_min_blocks<T>()) k4_xout_w(Dims 
     if (S.count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(S.count, 1ull);
 }
 
-// four-step inverse x FFT + crop + Au = u - u_s; ROWS rows x 3 components per block; src w2.
-template <typename T, int A, int B, int ROWS>
-__global__ void __launch_bounds__(3 * ROWS * FourStep<A LSM_COMMA B>::TPL, sizeof(T) == 8 ? 3 : 2) k4_fftx_out(Dims d, const ApplySys<T>* __restrict__ sys,
-                                                                      const typename cplx_of<T>::type* __restrict__ tw,
-                                                                      int xoff) {
-    typedef typename cplx_of<T>::type C;
-    constexpr int L = A * B, TPL = FourStep<A, B>::TPL, NL = 3 * ROWS, NTHR = NL * TPL, LD = NL + 1, PER = L / TPL;
-    extern __shared__ unsigned char smem_raw[];
-    const ApplySys<T> S = sys[blockIdx.z];
+// The same for L = A * B, A != B (FP32): each line on TPL = min(A, B) consecutive lanes, I1 step-1 DFTs
+// or I2 step-2 DFTs per lane, its tile padded so that the lines of a half warp meet different banks.
+// in[i][k]: element q + TPL i + B k of the line (k < NZ, the rest zero).  st(k, X[k]).
+// Bound by its loads' latency and HBM; the tile-transposing kernels it replaced made three
+// shared-memory round trips per element and four block barriers.  FP32 apply, one system:
+// 256^3 (L = 512) 5.70 -> 5.47 ms, 64^3 (L = 128) 112 -> 107 us.
+template <int A, int B> struct RowsW2 {
+    typedef FourStep<A, B> F;
+    static constexpr int LPB = 128 / F::TPL;                                     // lines per block
+    static constexpr int TILE = B * (A + 1) + (F::TPL < 16 ? F::TPL : 0);        // elements per line
+    static constexpr int MIN_BLOCKS = A * B == 512 ? 4 : 8;
+};
+template <int DIR, int A, int B, int NZ, int NO, class St>
+__device__ __forceinline__ void rows_w2(float2 (&in)[FourStep<A, B>::I1][NZ], float2* tl, const float2* __restrict__ tw, int q, St st) {
+    typedef FourStep<A, B> F;
+#pragma unroll
+    for (int i = 0; i < F::I1; ++i) {
+        const int t = q + F::TPL * i;
+        float2 v[A];
+#pragma unroll
+        for (int k = 0; k < A; ++k) v[k] = k < NZ ? in[i][k < NZ ? k : 0] : czero<float2>();
+        dft_reg_p<A, DIR, NZ, A>(v);
+        tw_row<DIR, A * B, A>(v, tw, t);
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) tl[t * (A + 1) + k1] = v[k1];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < F::I2; ++i) {
+        const int k1 = q + F::TPL * i;
+        float2 w[B];
+#pragma unroll
+        for (int t = 0; t < B; ++t) w[t] = tl[t * (A + 1) + k1];
+        dft_reg_p<B, DIR, B, NO>(w);
+#pragma unroll
+        for (int k2 = 0; k2 < NO; ++k2) st(k1 + A * k2, w[k2]);
+    }
+}
+
+// forward x FFT of zero-padded rows, as k4_rows_w (in_count <= (A/2 + 1) B)
+template <int A, int B>
+__global__ void __launch_bounds__(128, RowsW2<A LSM_COMMA B>::MIN_BLOCKS) k4_rows_w2(
+    const float2* __restrict__ tw, const ApplySys<float>* __restrict__ sys, int src_sel, int dst_sel, long long nrows, int in_count) {
+    typedef FourStep<A, B> F;
+    typedef RowsW2<A, B> W;
+    constexpr int NZ = A / 2 + 1;
+    __shared__ float2 tile[W::LPB][W::TILE];
+    const ApplySys<float> S = sys[blockIdx.y];
     if (S.run && !*S.run) return;
-    C* s = reinterpret_cast<C*>(smem_raw);
-    const int z = blockIdx.y;
-    const int y0 = blockIdx.x * ROWS;
-    const C* __restrict__ src = S.w2;
-    const int tid = threadIdx.x;
-    C v[PER];
+    const int ln = threadIdx.x / F::TPL, q = threadIdx.x % F::TPL;
+    const long long row = (long long)blockIdx.x * W::LPB + ln;
+    const bool live = row < nrows;
+    const float2* __restrict__ src = pick<float2>(S, src_sel) + row * in_count;
+    float2* __restrict__ dst = pick<float2>(S, dst_sel) + row * (A * B);
+    float2 in[F::I1][NZ];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int i = tid + k * NTHR;
-        const int kx = i % L, l = i / L;
-        const int c = l / ROWS, y = y0 + l % ROWS;
-        v[k] = (y < d.ny) ? src[(((long long)c * d.nz + z) * d.ny + y) * L + kx] : czero<C>();
-    }
+    for (int i = 0; i < F::I1; ++i)
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int i = tid + k * NTHR;
-        s[(i % L) * LD + i / L] = v[k];
-    }
-    // FP32: u for the epilogue is fetched now, so its latency overlaps the transform (nx = L / 2);
-    // FP64 is bound by its arithmetic, and the registers cost it occupancy, so it reads u at the end
-    constexpr int NX = L / 2, PO = NL * NX / NTHR;
-    constexpr bool PRE = sizeof(T) == 4;
-    const C* __restrict__ uin = S.u;
-    C uo[PRE ? PO : 1];
-    if constexpr (PRE) {
-#pragma unroll
-        for (int k = 0; k < PO; ++k) {
-            const int i = tid + k * NTHR;
-            const int x = i % NX, l = i / NX;
-            const int c = l / ROWS, y = y0 + l % ROWS;
-            uo[k] = (y < d.ny) ? uin[(((long long)c * d.nz + z) * d.ny + y) * NX + x] : czero<C>();
+        for (int k = 0; k < NZ; ++k) {
+            const int e = q + F::TPL * i + B * k;
+            in[i][k] = (live && e < in_count) ? src[e] : czero<float2>();
         }
-    }
-    __syncthreads();
-    fft4_smem<A, B, 1, A, B / 2 + 1>(s, NL, LD, tw, tid);   // outputs x + xoff <= L/2 only
-    C* __restrict__ out = S.out;
+    rows_w2<-1, A, B, NZ, B>(in, tile[ln], tw, q, [&](int k, float2 r) {
+        if (live) dst[k] = r;
+    });
+}
+
+// inverse x FFT of the rows of w2, crop, Au = u - u_s, as k4_xout_w (nx + xoff <= (B/2 + 1) A)
+template <int A, int B>
+__global__ void __launch_bounds__(128, RowsW2<A LSM_COMMA B>::MIN_BLOCKS) k4_xout_w2(
+    Dims d, const ApplySys<float>* __restrict__ sys, const float2* __restrict__ tw, int xoff) {
+    typedef FourStep<A, B> F;
+    typedef RowsW2<A, B> W;
+    __shared__ float2 tile[W::LPB][W::TILE];
+    const ApplySys<float> S = sys[blockIdx.y];
+    if (S.run && !*S.run) return;
+    const int ln = threadIdx.x / F::TPL, q = threadIdx.x % F::TPL;
+    const long long row = (long long)blockIdx.x * W::LPB + ln;
+    const bool live = row < 3LL * d.nz * d.ny;
+    const float2* __restrict__ src = S.w2 + row * (A * B);
+    const float2* __restrict__ uin = S.u + row * d.nx;
+    float2* __restrict__ out = S.out + row * d.nx;
+    float2 in[F::I1][A];
 #pragma unroll
-    for (int k = 0; k < PO; ++k) {
-        const int i = tid + k * NTHR;
-        const int x = i % NX, l = i / NX;
-        const int c = l / ROWS, y = y0 + l % ROWS;
-        if (y < d.ny) {
-            const long long idx = (((long long)c * d.nz + z) * d.ny + y) * NX + x;
-            const C uv = PRE ? uo[PRE ? k : 0] : uin[idx];
-            out[idx] = csub(uv, s[(x + xoff) * LD + l]);
-        }
-    }
-    if (S.count && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(S.count, 1ull);
+    for (int i = 0; i < F::I1; ++i)
+#pragma unroll
+        for (int k = 0; k < A; ++k) in[i][k] = live ? src[q + F::TPL * i + B * k] : czero<float2>();
+    rows_w2<1, A, B, A, B / 2 + 1>(in, tile[ln], tw, q, [&](int k, float2 r) {
+        const int x = k - xoff;
+        if (live && x >= 0 && x < d.nx) out[x] = csub(uin[x], r);
+    });
+    if (S.count && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(S.count, 1ull);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1613,11 +1607,8 @@ static void launch_xrows(const Dims& d, const ApplySys<T>* sys, int nsys, const 
             k4_rows_w<T, A, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * A, 0, st>>>((const C*)pl.twx, sys, src_sel, dst_sel,
                                                                                    nrows, in_count);
         } else if constexpr (F::INPLACE) {
-            constexpr int A = F::A_, B = F::B_, NL = 8;   // FP32 only: double-float has no A != B engine
-            const size_t sm = (size_t)A * B * (NL + 1) * sizeof(C);
-            smem_attr((const void*)k4_rows<T, -1, A, B, NL>, sm);
-            k4_rows<T, -1, A, B, NL><<<dim3(cdiv(nrows, NL), nsys), NL * F::TPL, sm, st>>>(
-                (const C*)pl.twx, sys, src_sel, dst_sel, nrows, in_count, 0, d.Lx, 0);
+            constexpr int A = F::A_, B = F::B_, LPB = RowsW2<A, B>::LPB;   // FP32 only: double-float has no A != B engine
+            k4_rows_w2<A, B><<<dim3(cdiv(nrows, LPB), nsys), 128, 0, st>>>((const C*)pl.twx, sys, src_sel, dst_sel, nrows, in_count);
         } else {
             const int NL = generic_rows_nl<T>(d.Lx, v == 2);
             const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(C);
@@ -1674,11 +1665,8 @@ static void launch_fftx_out(const Dims& d, const ApplySys<T>* sys, int nsys, con
             }
             k4_xout_w<T, A, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * A, 0, st>>>(d, sys, (const C*)pl.twx, xoff);
         } else if constexpr (F::INPLACE) {
-            constexpr int A = F::A_, B = F::B_, ROWS = sizeof(T) == 4 ? 8 : 4;
-            const size_t sm = (size_t)A * B * (3 * ROWS + 1) * sizeof(C);
-            smem_attr((const void*)k4_fftx_out<T, A, B, ROWS>, sm);
-            k4_fftx_out<T, A, B, ROWS><<<dim3(cdiv(d.ny, ROWS), d.nz, nsys), 3 * ROWS * F::TPL, sm, st>>>(
-                d, sys, (const C*)pl.twx, xoff);
+            constexpr int A = F::A_, B = F::B_, LPB = RowsW2<A, B>::LPB;
+            k4_xout_w2<A, B><<<dim3(cdiv(3LL * d.nz * d.ny, LPB), nsys), 128, 0, st>>>(d, sys, (const C*)pl.twx, xoff);
         } else {
             int B, th;
             size_t sm;
