@@ -1550,7 +1550,7 @@ constexpr size_t FX_STATIC_SM = 256;   // at least the fixed-point kernels' stat
 
 // Fixed-point tables of axis a, and the one the two-step plan of length L uses
 static inline FxTables fx_tables(const Plans& pl, int a) { return FxTables{pl.fx2[a], pl.fx3[a]}; }
-static inline const int4* fx_twostep(const Plans& pl, int a, int L) { return fx_prescale(L) == 2 ? pl.fx2[a] : pl.fx3[a]; }
+static inline const int4* fx_twostep(const Plans& pl, int a, int L) { return fx_twiddle_k(L) == 2 ? pl.fx2[a] : pl.fx3[a]; }
 
 // Width (lines) of a generic fixed-point tile: the widest of 8, 4, 2 (at most `most`) whose two buffers
 // fit `cap` bytes; half of it for schedule variant 2.  The z pass takes 4 columns up to L = 128 and 2

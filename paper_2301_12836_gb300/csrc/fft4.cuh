@@ -155,6 +155,63 @@ template <int S, int NZ, int NO, typename C> __device__ __forceinline__ void bfl
     }
 }
 
+// Fixed-point 32-point DFT times 1/4 (all inputs, first NO outputs), in two units.  Radix 8 over
+// the samples t = 4 a + b in the inputs' unit, products with W32^(b k) / 4 into a unit four times
+// coarser, and a last radix-4 layer of additions alone.  As 2 x 16 points in one unit (every inner
+// product rounded in the outputs' unit, which had to leave one bit more of headroom), an inverse
+// 512-point line of a Green-multiplied spectrum had 1.8 to 3.7 times the FP64 engine's error; it has
+// 0.49 to 0.88 of it.  256^3 FP64 apply 20.03 -> 20.09 ms.
+template <int S> __device__ __forceinline__ fxc fx_tw32_quarter(fxc a, int k) {
+    const double c[8] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                         0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173, 0.19509032201612826785};
+    const int q = k >> 3, j = k & 7;
+    if (j == 0) {   // +-1, +-i
+        const fxc r{fx_r((fx_ll(a.x) + 2) >> 2), fx_r((fx_ll(a.y) + 2) >> 2)};
+        return q == 0 ? r : cmul_si<S>(r);   // k < 22: 0 or 8 here
+    }
+    const long long kc = fx_const(c[j]), ks = fx_const(c[8 - j]);   // cos, sin(2 pi j / 32)
+    const long long re = q == 0 ? kc : (q == 1 ? -ks : -kc), im = q == 0 ? ks : (q == 1 ? kc : -ks);
+    return fx_cmul_quarter(a, re, S * im);
+}
+template <int S> __device__ __forceinline__ void fx_bfly8_wide(fxc* v) {   // bfly8 for sums below 2^62.6
+    const long long r2 = fx_const(0.70710678118654752440);
+    fxc e[4] = {v[0], v[2], v[4], v[6]};
+    fxc o[4] = {v[1], v[3], v[5], v[7]};
+    bfly4<S>(e);
+    bfly4<S>(o);
+    // o[1] (1 + S i) / sqrt2 and o[3] (-1 + S i) / sqrt2 from sums and differences
+    const fxr s1 = fx_scale_wide(fx_add(o[1].x, o[1].y), r2), d1 = fx_scale_wide(fx_sub(o[1].x, o[1].y), r2);
+    const fxr s3 = fx_scale_wide(fx_add(o[3].x, o[3].y), r2), d3 = fx_scale_wide(fx_sub(o[3].x, o[3].y), r2);
+    const fxc o1 = S > 0 ? fxc{d1, s1} : fxc{s1, fx_neg(d1)};
+    const fxc o3 = S > 0 ? fxc{fx_neg(s3), d3} : fxc{fx_neg(d3), fx_neg(s3)};
+    v[0] = cadd(e[0], o[0]);       v[4] = csub(e[0], o[0]);
+    v[1] = cadd(e[1], o1);         v[5] = csub(e[1], o1);
+    v[2] = fx_addi<S>(e[2], o[2]); v[6] = fx_subi<S>(e[2], o[2]);
+    v[3] = cadd(e[3], o3);         v[7] = csub(e[3], o3);
+}
+template <int S, int NZ, int NO> __device__ __forceinline__ void bfly32p(fxc* v) {
+    static_assert(NZ == 32 && (NO == 17 || NO == 32), "whole lines in, a cropped or a whole line out");
+    fxc y[4][8];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+#pragma unroll
+        for (int a = 0; a < 8; ++a) y[b][a] = v[4 * a + b];
+        fx_bfly8_wide<S>(y[b]);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        fxc z[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) z[b] = fx_tw32_quarter<S>(y[b][k], b * k);
+        if (NO == 32) bfly4p<S, 4, 4>(z);
+        else if (k == 0) bfly4p<S, 4, 3>(z);
+        else bfly4p<S, 4, 2>(z);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + 8 * j < NO) v[k + 8 * j] = z[j];
+    }
+}
+
 // R-point DFT with inputs NZ..R-1 zero and only the first NO outputs needed.  Pruned forms exist
 // for R = 32, 16 and 4 (and R = 8 with NZ <= 4, R = 2 with NZ = 1); otherwise the full DFT runs.
 template <int R, int S, int NZ, int NO, typename C> __device__ __forceinline__ void dft_reg_p(C* v) {

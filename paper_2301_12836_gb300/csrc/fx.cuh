@@ -5,10 +5,12 @@
 // product-and-sum 28.5).  A Fourier transform of one line has a known range (|X| <= the number of its
 // inputs times their largest modulus), so its FP64 transforms run here on integers: the line is
 // scaled by a power of two that leaves exactly that headroom, every butterfly addition is exact, and
-// only products round, to one unit of the last place.  The unit is 2^-54 to 2^-58 of the line's
-// largest input (FP64's own is 2^-53 of each value); against an 80-bit evaluation the operator's
-// normwise error measured 0.83 to 1.01 of the FP64 engine's on smooth, white, plane-wave and
-// point-source fields (grids with sides 16 to 128).  Inputs and outputs stay FP64 in memory.
+// only products round, to one unit of the last place.  The results' unit is 2^-57 (L = 16) to 2^-53
+// (inverse transforms of L = 512) of the line's largest input; the first step, and half of the
+// 32-point DFT, work in units 4 to 16 times finer.  (FP64's own unit is 2^-53 of each value.)  Against
+// longdouble a line's rms error is 0.16 to 1.0 of that of the same plan in FP64, in the worst of six
+// kinds of fields 0.88 on inverse lines at L = 512 (tests/test_fixed_point_lines.py).  Inputs and
+// outputs stay FP64 in memory.
 // Measured at 128^3, one system: FP64 apply 9.05 -> 2.13 ms (z pass 5.21 -> 0.93, y passes 1.05 -> 0.175
 // each, inverse x 0.57 -> 0.12, contrast source and forward x 0.76 -> 0.31).
 //
@@ -24,6 +26,7 @@
 // the twiddled values and the last butterflies' constants.
 #pragma once
 #include "common.cuh"
+#include <cmath>
 
 namespace lsm {
 
@@ -45,6 +48,8 @@ __host__ __device__ __forceinline__ fxr fx_r(long long v) {
     r.h = (int)(v >> 32);
     return r;
 }
+#ifdef __CUDACC__
+#define FX_RANGE(ok)
 __device__ __forceinline__ fxr fx_add(fxr a, fxr b) {
     fxr r;
     asm("add.cc.u32 %0, %2, %4; addc.u32 %1, %3, %5;" : "=r"(r.l), "=r"(r.h) : "r"(a.l), "r"(a.h), "r"(b.l), "r"(b.h));
@@ -55,7 +60,6 @@ __device__ __forceinline__ fxr fx_sub(fxr a, fxr b) {
     asm("sub.cc.u32 %0, %2, %4; subc.u32 %1, %3, %5;" : "=r"(r.l), "=r"(r.h) : "r"(a.l), "r"(a.h), "r"(b.l), "r"(b.h));
     return r;
 }
-__device__ __forceinline__ fxr fx_neg(fxr a) { return fx_sub(fxr{0u, 0}, a); }
 // a b + c.  As a product and a sum the assembler makes one multiply-add of it (28 per SM and clock, on
 // the FMA pipe alone); mad.wide.s32 came out as 2.5 instructions (23 per clock), and C as a 64 x 64
 // bit product where it knows an operand to be non-negative.
@@ -74,6 +78,30 @@ __device__ __forceinline__ fxr fx_words(long long v) {
     asm("mov.b64 {%0, %1}, %2;" : "=r"(r.l), "=r"(r.h) : "l"(v));
     return r;
 }
+#else
+// Host form, for tests of this arithmetic on the CPU: the same results, with every sum and every
+// factor's range checked.
+static long fx_range_errors = 0;
+#define FX_RANGE(ok) (fx_range_errors += !(ok))
+inline fxr fx_add(fxr a, fxr b) {
+    long long r;
+    FX_RANGE(!__builtin_add_overflow(fx_ll(a), fx_ll(b), &r));
+    return fx_r(r);
+}
+inline fxr fx_sub(fxr a, fxr b) {
+    long long r;
+    FX_RANGE(!__builtin_sub_overflow(fx_ll(a), fx_ll(b), &r));
+    return fx_r(r);
+}
+inline long long fx_mad(int a, int b, long long c) {
+    long long r;
+    FX_RANGE(!__builtin_add_overflow((long long)a * b, c, &r));
+    return r;
+}
+inline long long fx_pack(unsigned l, int h) { return fx_ll(fxr{l, h}); }
+inline fxr fx_words(long long v) { return fx_r(v); }
+#endif
+__device__ __forceinline__ fxr fx_neg(fxr a) { return fx_sub(fxr{0u, 0}, a); }
 __device__ __forceinline__ long long fx_sext(int h) { return fx_pack((unsigned)h, h >> 31); }
 template <> __device__ __forceinline__ fxc cadd<fxc>(fxc a, fxc b) { return fxc{fx_add(a.x, b.x), fx_add(a.y, b.y)}; }
 template <> __device__ __forceinline__ fxc csub<fxc>(fxc a, fxc b) { return fxc{fx_sub(a.x, b.x), fx_sub(a.y, b.y)}; }
@@ -116,6 +144,7 @@ __host__ __device__ __forceinline__ constexpr long long fx_const(double c) {
 
 // v = h 2^32 + l with l signed
 __device__ __forceinline__ void fx_split(fxr v, int& h, int& l) {
+    FX_RANGE(fx_ll(v) < 0x7fffffff80000000LL);
     l = (int)v.l;
     h = v.h + (int)(v.l >> 31);
 }
@@ -125,6 +154,7 @@ __host__ __device__ __forceinline__ constexpr int fx_w0(long long k) {
 }
 // v k 2^-62 (|v| < 2^62)
 __device__ __forceinline__ fxr fx_scale(fxr v, long long k) {
+    FX_RANGE(fx_ll(v) >> 62 == fx_ll(v) >> 63);
     const int v1 = fx_sr31w(v), v0 = (int)(v.l & 0x7fffffffu);
     const int w1 = fx_w1(k), w0 = fx_w0(k);
     const long long t = fx_mad(v1, w0, fx_mad(v0, w1, 1LL << 30));
@@ -132,6 +162,7 @@ __device__ __forceinline__ fxr fx_scale(fxr v, long long k) {
 }
 // a (re + i im), re = r1 2^-31 + r0 2^-62 and so im (|a| < 2^60.67)
 __device__ __forceinline__ fxc fx_cmul(fxc a, int r1, int r0, int i1, int i0) {
+    FX_RANGE(fx_ll(a.x) >> 62 == fx_ll(a.x) >> 63 && fx_ll(a.y) >> 62 == fx_ll(a.y) >> 63);
     const int x1 = fx_sr31w(a.x), x0 = (int)(a.x.l & 0x7fffffffu);
     const int y1 = fx_sr31w(a.y), y0 = (int)(a.y.l & 0x7fffffffu);
     const long long tr = fx_mad(y1, -i0, fx_mad(y0, -i1, fx_mad(x1, r0, fx_mad(x0, r1, 1LL << 30))));
@@ -148,6 +179,19 @@ __device__ __forceinline__ fxc fx_cmul32(fxc a, int r1, int r0, int i1, int i0) 
     const fxr tr = fx_words(fx_mad(yh, -i0, fx_mad(yl, -i1, fx_mad(xh, r0, fx_mad(xl, r1, 1LL << 31)))));
     const fxr ti = fx_words(fx_mad(yh, r0, fx_mad(yl, r1, fx_mad(xh, i0, fx_mad(xl, i1, 1LL << 31)))));
     return fxc{fx_words(fx_mad(yh, -i1, fx_mad(xh, r1, fx_sext(tr.h)))), fx_words(fx_mad(yh, r1, fx_mad(xh, i1, fx_sext(ti.h))))};
+}
+// v k 2^-62 for |v| < 2^63, one more multiply-add (k < 2^62 a constant whose low word is below 2^30)
+__device__ __forceinline__ fxr fx_scale_wide(fxr v, long long k) {
+    int h, l;
+    fx_split(v, h, l);
+    const int k1 = fx_w1(k), k0 = 2 * fx_w0(k);
+    const long long t = fx_mad(h, k0, fx_mad(l, k1, 1LL << 30));
+    return fx_words(fx_mad(h, k1, fx_mad(h, k1, fx_sr31(t))));
+}
+// a (re + i im) / 4, re = kr 2^-62 and so im, |re + i im| = 1 (|a| < 2^62.7)
+__device__ __forceinline__ fxc fx_cmul_quarter(fxc a, long long kr, long long ki) {
+    const int r1 = (int)((kr + (1LL << 31)) >> 32), i1 = (int)((ki + (1LL << 31)) >> 32);
+    return fx_cmul32(a, r1, (int)(kr - ((long long)r1 << 32)), i1, (int)(ki - ((long long)i1 << 32)));
 }
 // v 2^-sh, rounded to nearest, for sh of either sign; 64 or more shifts any value out
 __device__ __forceinline__ fxr fx_shift(fxr v, int sh) {
@@ -178,13 +222,28 @@ template <int S, typename C> __device__ __forceinline__ C tw_mul(C a, const C* _
     return cmul(a, w);
 }
 template <int S> __device__ __forceinline__ fxc tw_mul32(fxc a, const int4* __restrict__ tw, int k) {
+#ifdef __CUDACC__
     // volatile: 15 entries fetched ahead of their use would spill
     int4 w;
     asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(tw + k));
+#else
+    const int4 w = tw[k];
+#endif
     return S > 0 ? fx_cmul32(a, w.x, w.y, -w.z, -w.w) : fx_cmul32(a, w.x, w.y, w.z, w.w);
 }
-// K of the two-step plan of length L
-__host__ __device__ constexpr int fx_prescale(int L) { return L == 16 ? 2 : 3; }
+// v (|v| <= 1/4) as the two-word fixed-point number v1 2^-32 + v0 2^-64, v0 within +-(2^31 - 1) so
+// that either sign can be negated
+inline void fx_table_words(long double v, int* v1, int* v0) {
+    const long double f = 4294967296.0L, lim = 2147483647.0L;
+    const long double a = nearbyintl(v * f);
+    const long double b = nearbyintl((v * f - a) * f);
+    *v1 = (int)a;
+    *v0 = (int)(b > lim ? lim : (b < -lim ? -lim : b));
+}
+// K of the two-step plan of length L, and the part of it that the twiddles between the steps carry
+// (L = 512: the second step is the 32-point DFT in two units, which carries the other 2)
+__host__ __device__ constexpr int fx_prescale(int L) { return L == 16 ? 2 : (L == 512 ? 4 : 3); }
+__host__ __device__ constexpr int fx_twiddle_k(int L) { return L == 16 || L == 512 ? 2 : 3; }
 
 // twiddles between the steps of a two-step transform of length L: v[k1] tw[t k1].  Row t = 0 has
 // none; in fixed point every entry also passes to the second step's unit (the table's entries carry
@@ -196,7 +255,7 @@ template <int S, int L, int A, typename C> __device__ __forceinline__ void tw_ro
     }
 }
 template <int S, int L, int A> __device__ __forceinline__ void tw_row(fxc* v, const int4* __restrict__ tw, int t) {
-    constexpr int K = fx_prescale(L);
+    constexpr int K = fx_twiddle_k(L);
     v[0].x = fx_r((fx_ll(v[0].x) + (1 << (K - 1))) >> K);
     v[0].y = fx_r((fx_ll(v[0].y) + (1 << (K - 1))) >> K);
 #pragma unroll
@@ -281,14 +340,14 @@ __device__ __forceinline__ double2 fx_to_odd(fxc v, const FxUnit& u) { return ma
 
 // Bits of a line's inputs, in the unit of the outputs: a line with at most nin nonzero inputs, each
 // component below 2^bits in modulus, keeps its outputs below 2^62.6 (log2(nin) + 1/2 bits of growth).
-// last: radix of the last step's DFT; 8 and 32 multiply just before their final additions, so one
-// bit less keeps those products' factors in range.  nz: nonzero
-// inputs of a first-step DFT, whose outputs, 2^K finer, stay below 2^61.9.
+// last: radix of the last step's DFT; 8 multiplies just before its final additions, so one bit less
+// keeps those products' factors in range.  nz: nonzero inputs of a first-step DFT, whose outputs, 2^K
+// finer, stay below 2^61.9.
 inline int fx_bits(int L, int nin, int nz, int last) {
     const double one = 4611686018427387904.0;   // 2^62
     int b = 62;
     while (b > 0 && (double)nin * (double)(1ull << b) > 1.0717734625362931 * one) --b;   // 2^62.1
-    if (last == 8 || last == 32) --b;
+    if (last == 8) --b;
     while (b > 0 && (double)nz * (double)(1ull << b) * (1 << fx_prescale(L)) > 0.6597539553864471 * one) --b;   // 2^61.4
     return b;
 }

@@ -181,16 +181,6 @@ bool factor_plan(int L, FxPlan& p) {
     return m == 1;
 }
 
-// v (|v| <= 1/4) as the two-word fixed-point number v1 2^-32 + v0 2^-64, v0 within +-(2^31 - 1) so
-// that either sign can be negated
-void fx_table_words(long double v, int* v1, int* v0) {
-    const long double f = 4294967296.0L, lim = 2147483647.0L;
-    const long double a = nearbyintl(v * f);
-    const long double b = nearbyintl((v * f - a) * f);
-    *v1 = (int)a;
-    *v0 = (int)(b > lim ? lim : (b < -lim ? -lim : b));
-}
-
 // exp(-2 pi i k / L), k < L, evaluated in long double and rounded once; fx2, fx3: as fixed-point words
 // times 2^-2 and 2^-3
 void twiddle_table(int L, std::vector<double2>& t64, std::vector<float2>& t32, std::vector<int4>& fx2, std::vector<int4>& fx3) {
