@@ -1562,22 +1562,35 @@ static inline int fxg_width(int L, int per, int most, size_t cap, int v) {
     if (v == 2 && w > 2) w /= 2;
     return w;
 }
-template <typename Fn> static void with_width(int w, Fn&& fn) {
-    if (w == 8) fn(std::integral_constant<int, 8>());
-    else if (w == 4) fn(std::integral_constant<int, 4>());
-    else fn(std::integral_constant<int, 2>());
+// Call fn with the width and the plan's kind as constants: 8 or 4 lines, or 2 for the half tile of lines
+// too long for 8, which are all dynamic ones; z passes 4 columns or 2, dynamic plans (L > 128) 2.
+template <typename Fn> static void with_tile(int w, const FxPlan& p, Fn&& fn) {
+    using std::integral_constant;
+    if (!p.fxdyn) {
+        if (w == 8) fn(integral_constant<int, 8>(), std::false_type());
+        else fn(integral_constant<int, 4>(), std::false_type());
+    } else if (w == 8) fn(integral_constant<int, 8>(), std::true_type());
+    else if (w == 4) fn(integral_constant<int, 4>(), std::true_type());
+    else fn(integral_constant<int, 2>(), std::true_type());
+}
+template <typename Fn> static void with_ztile(int w, const FxPlan& p, Fn&& fn) {
+    using std::integral_constant;
+    if (p.fxdyn) fn(integral_constant<int, 2>(), std::true_type());
+    else if (w == 4) fn(integral_constant<int, 4>(), std::false_type());
+    else fn(integral_constant<int, 2>(), std::false_type());
 }
 
 // FP64 rows through the generic fixed-point engine; OUT as in kg_rows_fx
 template <int DIR, bool OUT>
 static void launch_rows_fxg(const Dims& d, const ApplySys<double>* sys, int nsys, const Plans& pl, int src_sel, int dst_sel,
                             long long nrows, int in_count, int in_off, int out_count, int out_off, cudaStream_t st, int v) {
-    with_width(fxg_width(d.Lx, 1, 8, SMEM_CAP, v), [&](auto w) {
+    with_tile(fxg_width(d.Lx, 1, 8, SMEM_CAP, v), pl.px, [&](auto w, auto dyn) {
         constexpr int NL = decltype(w)::value;
+        constexpr bool DYN = decltype(dyn)::value;
         const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(fxc);
         const int m = fxg_groups(pl.px, 64 / NL, NL < 4 ? 48 : 192 / NL);
-        smem_attr((const void*)kg_rows_fx<DIR, NL, OUT>, sm, FX_STATIC_SM);
-        kg_rows_fx<DIR, NL, OUT><<<dim3(cdiv(nrows, NL), nsys), NL * m, sm, st>>>(
+        smem_attr((const void*)kg_rows_fx<DIR, NL, OUT, DYN>, sm, FX_STATIC_SM);
+        kg_rows_fx<DIR, NL, OUT, DYN><<<dim3(cdiv(nrows, NL), nsys), NL * m, sm, st>>>(
             pl.px, fx_tables(pl, 0), sys, src_sel, dst_sel, nrows, in_count, in_off, out_count, out_off);
     });
 }
@@ -1694,12 +1707,13 @@ static void launch_strided(int L, const FxPlan& p, const void* tw, const Plans& 
                 k4_strided_fx<DIR, A, B, TXC><<<dim3(cdiv(a.nlines, TXC), outer, a.ncomp * nsys), TXC * F::TPL, sm, st>>>(
                     fx_twostep(pl, axis, L), a, sys, fx_bits(L, a.in_count, DIR < 0 ? A / 2 + 1 : A, B));
             } else {
-                with_width(fxg_width(L, 1, 8, SMEM_CAP, v), [&](auto w) {
+                with_tile(fxg_width(L, 1, 8, SMEM_CAP, v), p, [&](auto w, auto dyn) {
                     constexpr int NL = decltype(w)::value;
+                    constexpr bool DYN = decltype(dyn)::value;
                     const size_t sm = 2 * (size_t)L * NL * sizeof(fxc);
                     const int m = fxg_groups(p, 64 / NL, NL < 4 ? 48 : 192 / NL);
-                    smem_attr((const void*)kg_strided_fx<DIR, NL>, sm, FX_STATIC_SM);
-                    kg_strided_fx<DIR, NL><<<dim3(cdiv(a.nlines, NL), outer, a.ncomp * nsys), NL * m, sm, st>>>(
+                    smem_attr((const void*)kg_strided_fx<DIR, NL, DYN>, sm, FX_STATIC_SM);
+                    kg_strided_fx<DIR, NL, DYN><<<dim3(cdiv(a.nlines, NL), outer, a.ncomp * nsys), NL * m, sm, st>>>(
                         p, fx_tables(pl, axis), a, sys);
                 });
             }
@@ -1766,12 +1780,13 @@ static void launch_zpass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
                     d, fx_twostep(pl, 2, A * B), sys, nsys, in_count, in_off, out_count, out_off, src_sel, dst_sel,
                     fx_bits(A * B, in_count, A / 2 + 1, B), fx_bits(A * B, A * B, A, B));
             } else {
-                with_width(fxg_width(d.Lz, 3, d.Lz > 128 ? 2 : 4, SMEM_CAP, v), [&](auto w) {
+                with_ztile(fxg_width(d.Lz, 3, d.Lz > 128 ? 2 : 4, SMEM_CAP, v), pl.pz, [&](auto w, auto dyn) {
                     constexpr int TXC = decltype(w)::value, NL = 3 * TXC;
+                    constexpr bool DYN = decltype(dyn)::value;
                     const size_t smf = (size_t)d.Lz * (2 * NL * sizeof(fxc) + TXC * sizeof(int));
                     const int m = fxg_groups(pl.pz, 8, NL < 8 ? 32 : 192 / NL);
-                    smem_attr((const void*)kg_fftz_green_fx<CONJ, TXC>, smf, FX_STATIC_SM);
-                    kg_fftz_green_fx<CONJ, TXC><<<dim3(cdiv(d.Lx, TXC) * nsys, d.Ly, 1), NL * m, smf, st>>>(
+                    smem_attr((const void*)kg_fftz_green_fx<CONJ, TXC, DYN>, smf, FX_STATIC_SM);
+                    kg_fftz_green_fx<CONJ, TXC, DYN><<<dim3(cdiv(d.Lx, TXC) * nsys, d.Ly, 1), NL * m, smf, st>>>(
                         d, pl.pz, fx_tables(pl, 2), sys, nsys, in_count, in_off, out_count, out_off, src_sel, dst_sel);
                 });
             }
@@ -2200,17 +2215,18 @@ cudaError_t launch_octant_fft(const Dims& d, const Plans& pl, double2* buf, cuda
         if (a == 0) { s.ls = sx; s.es = 1; s.os = 0; s.nlines = (int)(sy * sz); }
         else if (a == 1) { s.ls = 1; s.es = sx; s.os = sx * sy; s.nlines = (int)sx; outer = (int)sz; }
         else { s.ls = 1; s.es = sx * sy; s.os = 0; s.nlines = (int)(sx * sy); }
-        with_width(fxg_width(p[a]->L, 1, 8, SMEM_CAP, 0), [&](auto w) {
+        with_tile(fxg_width(p[a]->L, 1, 8, SMEM_CAP, 0), *p[a], [&](auto w, auto dyn) {
             constexpr int NL = decltype(w)::value;
+            constexpr bool DYN = decltype(dyn)::value;
             const int m = fxg_groups(*p[a], 64 / NL, NL < 4 ? 48 : 192 / NL);
             const size_t sm = 2 * (size_t)p[a]->L * (NL + (a == 0)) * sizeof(fxc);
             const dim3 grid(cdiv(s.nlines, NL), outer, 6);
             if (a == 0) {
-                smem_attr((const void*)kg_sym_fx<NL, true>, sm, FX_STATIC_SM);
-                kg_sym_fx<NL, true><<<grid, NL * m, sm, st>>>(*p[a], fx_tables(pl, a), s, buf);
+                smem_attr((const void*)kg_sym_fx<NL, true, DYN>, sm, FX_STATIC_SM);
+                kg_sym_fx<NL, true, DYN><<<grid, NL * m, sm, st>>>(*p[a], fx_tables(pl, a), s, buf);
             } else {
-                smem_attr((const void*)kg_sym_fx<NL, false>, sm, FX_STATIC_SM);
-                kg_sym_fx<NL, false><<<grid, NL * m, sm, st>>>(*p[a], fx_tables(pl, a), s, buf);
+                smem_attr((const void*)kg_sym_fx<NL, false, DYN>, sm, FX_STATIC_SM);
+                kg_sym_fx<NL, false, DYN><<<grid, NL * m, sm, st>>>(*p[a], fx_tables(pl, a), s, buf);
             }
         });
     }

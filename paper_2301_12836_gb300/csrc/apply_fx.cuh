@@ -252,10 +252,6 @@ __device__ __forceinline__ fxc fx_gdot3(const int4& g0, const FxQ& qa, const int
     fx_gmac<CONJ>(g2, qc, hr, tr, hi, ti);
     return fxc{fx_add(fx_words(hr), fx_sr30(tr)), fx_add(fx_words(hi), fx_sr30(ti))};
 }
-__device__ __forceinline__ unsigned fx_hibits(fxc v) {
-    return (unsigned)((v.x.h ^ (v.x.h >> 31)) | (v.y.h ^ (v.y.h >> 31)));
-}
-
 constexpr int FX_NO_KEY = -(1 << 24);   // below any exponent
 
 // Maximum over the lanes of each aligned group of 16 whose numbers agree modulo TX (the same column

@@ -1,99 +1,18 @@
-// apply_fxg.cuh - the FP64 operator's transform passes in 64-bit fixed point (fx.cuh) for any line
-// length with factors 2, 3 and 5 (and for the two-step lengths on request of the schedule).
-// Included by apply.cu after apply_fx.cuh.
+// apply_fxg.cuh - the FP64 operator's transform passes in 64-bit fixed point for any line length with
+// factors 2, 3 and 5 (and for the two-step lengths on request of the schedule), on the runtime stages
+// of fxg.cuh.  Included by apply.cu after apply_fx.cuh.
 //
-// Runtime mixed-radix Stockham stages (fft.cuh) between two shared-memory buffers.  A thread keeps
-// one line (l) and one of m groups of butterflies (g), so no stage divides by the tile's width; m is
-// chosen on the host so that the groups fill every stage's butterflies as evenly as they can
-// (fxg_groups).  Every stage after the first carries 2^-K in its twiddles, K = 1 .. 3 such that all
-// stages keep the same range (chosen with the plan): a line's error is that of its last stages (K = 2
-// or 3 by the radix alone lost up to 3 bits on lines such as 250 = 2 5 5 5: error 1.6 of the FP64
-// engine's, now 0.9 to 0.99).
+// A thread keeps one line (l) and one of m groups of butterflies (g), so no stage divides by the tile's
+// width; m is chosen on the host so that the groups fill every stage's butterflies as evenly as they
+// can (fxg_groups).
 //
 // Bound by latency and the integer pipes (z pass at 96^3: issue 31% at 10 warps before the tile was
 // halved).  One system, FP64 apply: 96^3 4.62 -> 1.44 ms (z pass 2.74 -> 0.65, y 0.51 -> 0.14 each, inverse x
 // 0.30 -> 0.12), 60 x 45 x 50 0.92 -> 0.30 ms.
 #pragma once
+#include "fxg.cuh"
 
 namespace lsm {
-
-// the two scaled twiddle tables of a line length: entries times 2^-2 and 2^-3
-struct FxTables {
-    const int4 *t2, *t3;
-};
-
-template <int S, int R, int LD>
-__device__ __forceinline__ void fxg_stage(const fxc* __restrict__ src, fxc* __restrict__ dst, int L, int Ns, int K,
-                                          const FxTables& T, int l, int g, int m) {
-    const int4* __restrict__ tw = K == 3 ? T.t3 : T.t2;
-    const int nb = L / R, tstep = L / (Ns * R);
-    const unsigned magic = 0xffffffffu / (unsigned)Ns + 1;   // j / Ns = j magic 2^-32 for j < 2^16 (Ns > 1)
-#pragma unroll 1
-    for (int j = g; j < nb; j += m) {
-        const int jq = Ns == 1 ? j : (int)__umulhi((unsigned)j, magic);
-        const int k = j - jq * Ns;
-        fxc v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = src[(j + r * nb) * LD + l];
-        if (K) {   // not the first stage
-            v[0].x = fx_r((fx_ll(v[0].x) + (1 << (K - 1))) >> K);
-            v[0].y = fx_r((fx_ll(v[0].y) + (1 << (K - 1))) >> K);
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                if (K == 1) v[r] = cadd(v[r], v[r]);
-                v[r] = tw_mul32<S>(v[r], tw, r * k * tstep);
-            }
-        }
-        if constexpr (R == 2) bfly2<S>(v);
-        else if constexpr (R == 3) bfly3<S>(v);
-        else if constexpr (R == 4) bfly4<S>(v);
-        else if constexpr (R == 5) bfly5<S>(v);
-        else bfly8<S>(v);
-        const int base = jq * Ns * R + k;
-#pragma unroll
-        for (int r = 0; r < R; ++r) dst[(base + r * Ns) * LD + l] = v[r];
-    }
-}
-
-// Transform the tile in a (layout a[e * LD + l]); b is scratch of the same size.  Returns the buffer
-// of the result.  The caller synchronises before; the result is visible to the block on return.
-template <int S, int LD>
-__device__ __forceinline__ fxc* fxg_fft(fxc* a, fxc* b, const FxPlan& p, const FxTables& T, int l, int g, int m) {
-    int Ns = 1;
-    for (int s = 0; s < p.nst; ++s) {
-        const int R = p.radix[s];
-        switch (R) {
-            case 8: fxg_stage<S, 8, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
-            case 4: fxg_stage<S, 4, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
-            case 2: fxg_stage<S, 2, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
-            case 3: fxg_stage<S, 3, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
-            default: fxg_stage<S, 5, LD>(a, b, p.L, Ns, p.fxk[s], T, l, g, m); break;
-        }
-        __syncthreads();
-        fxc* t = a; a = b; b = t;
-        Ns *= R;
-    }
-    return a;
-}
-
-// Groups per line, m <= most: the fewest butterfly rounds weighted by their size, then the most groups.
-static inline int fxg_groups(const FxPlan& p, int least, int most) {
-    int best = least;
-    double cost = 1e300;
-    for (int m = least; m <= most; ++m) {
-        double c = 0.0;
-        for (int s = 0; s < p.nst; ++s) {
-            const int nb = p.L / p.radix[s];
-            c += (double)((nb + m - 1) / m) * (p.radix[s] + 2) * m;
-        }
-        c *= 1.0 + 4.0 / m;   // fewer threads hide less latency
-        if (c <= cost) {
-            cost = c;
-            best = m;
-        }
-    }
-    return best;
-}
 
 // Elements g, g + m, ... below n of a line, ld(e) -> raw[e * LD + l], four loads in flight; returns the
 // largest magnitude word.
@@ -115,10 +34,10 @@ __device__ __forceinline__ unsigned fxg_load(double2* raw, int n, int l, int g, 
 }
 
 // ---- strided pass: NL consecutive lines along x per block
-template <int DIR, int NL>
+template <int DIR, int NL, bool DYN>
 __global__ void __launch_bounds__(NL * 48) kg_strided_fx(FxPlan p, FxTables T, StridedArgs a, const ApplySys<double>* __restrict__ sys) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ unsigned s_mag[NL];
+    __shared__ unsigned s_mag[NL], s_hi[DYN ? 3 * NL : 1];
     const ApplySys<double>& S = sys[blockIdx.z / a.ncomp];
     if (S.run && !*S.run) return;
     const int c = blockIdx.z % a.ncomp;
@@ -131,6 +50,7 @@ __global__ void __launch_bounds__(NL * 48) kg_strided_fx(FxPlan p, FxTables T, S
     fxc* sb = sa + (size_t)p.L * NL;
     double2* raw = reinterpret_cast<double2*>(sb);
     if (threadIdx.x < NL) s_mag[threadIdx.x] = 0;
+    if (DYN && threadIdx.x < 3 * NL) s_hi[threadIdx.x] = 0;
     __syncthreads();
     const unsigned mag = fxg_load<NL>(raw, a.in_count, l, g, m, [&](int e) { return xin ? src[(long long)e * a.src_es] : czero<double2>(); });
     atomicMax(&s_mag[l], mag);
@@ -141,8 +61,9 @@ __global__ void __launch_bounds__(NL * 48) kg_strided_fx(FxPlan p, FxTables T, S
         sa[e * NL + l] = (es >= 0 && es < a.in_count) ? fx_from(raw[es * NL + l], sc, p.fxbits) : czero<fxc>();
     }
     __syncthreads();
-    const fxc* r = fxg_fft<DIR, NL>(sa, sb, p, T, l, g, m);
-    const FxUnit un(sc.unit(p.fxbits) + p.fxsum, sc.bad, s_mag[l] == 0);
+    int esum;
+    const fxc* r = fxg_fft<DIR, NL, DYN, NL>(sa, sb, p, T, l, g, m, s_hi, l, esum);
+    const FxUnit un(sc.unit(p.fxbits) + esum, sc.bad, s_mag[l] == 0);
     if (xin)
         for (int eo = g; eo < a.out_count; eo += m) {
             const fxc v = r[(eo + a.out_off) * NL + l];
@@ -152,13 +73,14 @@ __global__ void __launch_bounds__(NL * 48) kg_strided_fx(FxPlan p, FxTables T, S
 
 // ---- contiguous rows: NL rows per block.  Row r of src holds in_count elements (placed at in_off),
 // row r of dst out_count (from out_off).  OUT: the inverse x pass's epilogue, dst = S.out = u - result.
-template <int DIR, int NL, bool OUT>
+template <int DIR, int NL, bool OUT, bool DYN>
 __global__ void __launch_bounds__(NL * 48) kg_rows_fx(FxPlan p, FxTables T, const ApplySys<double>* __restrict__ sys, int src_sel,
                                                       int dst_sel, long long nrows, int in_count, int in_off, int out_count,
                                                       int out_off) {
     constexpr int LD = NL + 1;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ unsigned s_mag[NL];
+    __shared__ unsigned s_mag[NL], s_hi[DYN ? 3 * NL : 1];
+    __shared__ int s_sum[NL];
     const ApplySys<double>& S = sys[blockIdx.y];
     if (S.run && !*S.run) return;
     const int l = threadIdx.x % NL, g = threadIdx.x / NL, m = blockDim.x / NL;
@@ -171,6 +93,7 @@ __global__ void __launch_bounds__(NL * 48) kg_rows_fx(FxPlan p, FxTables T, cons
     fxc* sb = sa + (size_t)p.L * LD;
     double2* raw = reinterpret_cast<double2*>(sb);
     if (threadIdx.x < NL) s_mag[threadIdx.x] = 0;
+    if (DYN && threadIdx.x < 3 * NL) s_hi[threadIdx.x] = 0;
     __syncthreads();
     for (int k = 0; k < live; ++k) {
         unsigned mag = 0;
@@ -188,10 +111,15 @@ __global__ void __launch_bounds__(NL * 48) kg_rows_fx(FxPlan p, FxTables T, cons
         sa[e * LD + l] = (l < live && es >= 0 && es < in_count) ? fx_from(raw[es * LD + l], sc, p.fxbits) : czero<fxc>();
     }
     __syncthreads();
-    const fxc* r = fxg_fft<DIR, LD>(sa, sb, p, T, l, g, m);
+    int esum;
+    const fxc* r = fxg_fft<DIR, LD, DYN, NL>(sa, sb, p, T, l, g, m, s_hi, l, esum);
+    if constexpr (DYN) {
+        if (g == 0) s_sum[l] = esum;
+        __syncthreads();
+    }
     for (int k = 0; k < live; ++k) {
         const FxScale sk(s_mag[k]);
-        const FxUnit un(sk.unit(p.fxbits) + p.fxsum, sk.bad, s_mag[k] == 0);
+        const FxUnit un(sk.unit(p.fxbits) + (DYN ? s_sum[k] : esum), sk.bad, s_mag[k] == 0);
         for (int e = threadIdx.x; e < out_count; e += blockDim.x) {
             const fxc v = r[(e + out_off) * LD + k];
             const double2 w = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
@@ -203,13 +131,13 @@ __global__ void __launch_bounds__(NL * 48) kg_rows_fx(FxPlan p, FxTables T, cons
 }
 
 // ---- z pass with the Green multiply: TX columns of one ky, as k4_fftz_green_fx
-template <bool CONJ, int TX>
+template <bool CONJ, int TX, bool DYN>
 __global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FxPlan p, FxTables T, const ApplySys<double>* __restrict__ sys,
                                                                 int nsys, int in_count, int in_off, int out_count, int out_off,
                                                                 int src_sel, int dst_sel) {
     constexpr int NL = 3 * TX;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ unsigned s_mag[TX];
+    __shared__ unsigned s_mag[TX], s_hi[DYN ? 3 * TX : 1];
     __shared__ int s_key[TX];
     const ApplySys<double>& S = sys[blockIdx.x % nsys];
     if (S.run && !*S.run) return;
@@ -227,6 +155,7 @@ __global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FxPlan p
         s_mag[threadIdx.x] = 0;
         s_key[threadIdx.x] = FX_NO_KEY;
     }
+    if (DYN && threadIdx.x < 3 * TX) s_hi[threadIdx.x] = 0;
     __syncthreads();
     {
         const double2* __restrict__ src = pick<double2>(S, src_sel) + (size_t)cl * in_count * plane + col;
@@ -240,8 +169,10 @@ __global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FxPlan p
         sa[e * NL + l] = (es >= 0 && es < in_count) ? fx_from(raw[es * NL + l], sc, p.fxbits) : czero<fxc>();
     }
     __syncthreads();
-    fxc* s = fxg_fft<-1, NL>(sa, sb, p, T, l, g, m);
+    int esum, esum_inv;
+    fxc* s = fxg_fft<-1, NL, DYN, TX>(sa, sb, p, T, l, g, m, s_hi, lx, esum);   // one unit per column: its components mix
     fxc* o = s == sa ? sb : sa;
+    if (DYN && threadIdx.x < 3 * TX) s_hi[threadIdx.x] = 0;   // ordered before its use by the barrier after the multiply
     // ---- Green multiply
     {
         const int cx = threadIdx.x % TX, kx = x0 + cx;   // blockDim.x is a multiple of TX
@@ -294,8 +225,8 @@ __global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FxPlan p
         s[e * NL + l] = fxc{fx_shift(v.x, sh), fx_shift(v.y, sh)};
     }
     __syncthreads();
-    const fxc* r = fxg_fft<1, NL>(s, o, p, T, l, g, m);
-    const FxUnit un(sc.unit(p.fxbits) + 2 * p.fxsum + ecom, sc.bad || top > FxG::BAD_EXP / 2, s_mag[lx] == 0);
+    const fxc* r = fxg_fft<1, NL, DYN, TX>(s, o, p, T, l, g, m, s_hi, lx, esum_inv);
+    const FxUnit un(sc.unit(p.fxbits) + esum + esum_inv + ecom, sc.bad || top > FxG::BAD_EXP / 2, s_mag[lx] == 0);
     if (xin) {
         double2* __restrict__ dst = pick<double2>(S, dst_sel) + (size_t)cl * out_count * plane + col;
         for (int eo = g; eo < out_count; eo += m) {
@@ -314,11 +245,12 @@ struct SymArgs {
     long long cs, os, ls, es;
     int nlines, odd;
 };
-template <int NL, bool ROWS>
+template <int NL, bool ROWS, bool DYN>
 __global__ void __launch_bounds__(NL * 48) kg_sym_fx(FxPlan p, FxTables T, SymArgs a, double2* __restrict__ buf) {
     constexpr int LD = ROWS ? NL + 1 : NL;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ unsigned s_mag[NL];
+    __shared__ unsigned s_mag[NL], s_hi[DYN ? 3 * NL : 1];
+    __shared__ int s_sum[NL];
     const int n = p.L / 2, i0 = blockIdx.x * NL;
     const int l = threadIdx.x % NL, g = threadIdx.x / NL, m = blockDim.x / NL;
     const int live = a.nlines - i0 < NL ? a.nlines - i0 : NL;
@@ -327,6 +259,7 @@ __global__ void __launch_bounds__(NL * 48) kg_sym_fx(FxPlan p, FxTables T, SymAr
     fxc* sb = sa + (size_t)p.L * LD;
     double2* raw = reinterpret_cast<double2*>(sb);
     if (threadIdx.x < NL) s_mag[threadIdx.x] = 0;
+    if (DYN && threadIdx.x < 3 * NL) s_hi[threadIdx.x] = 0;
     __syncthreads();
     if constexpr (ROWS) {
         for (int k = 0; k < live; ++k) {
@@ -352,18 +285,23 @@ __global__ void __launch_bounds__(NL * 48) kg_sym_fx(FxPlan p, FxTables T, SymAr
             sa[e * LD + l] = v;
         }
     __syncthreads();
-    const fxc* r = fxg_fft<-1, LD>(sa, sb, p, T, l, g, m);
+    int esum;
+    const fxc* r = fxg_fft<-1, LD, DYN, NL>(sa, sb, p, T, l, g, m, s_hi, l, esum);
     if constexpr (ROWS) {
+        if constexpr (DYN) {
+            if (g == 0) s_sum[l] = esum;
+            __syncthreads();
+        }
         for (int k = 0; k < live; ++k) {
             const FxScale sk(s_mag[k]);
-            const FxUnit un(sk.unit(p.fxbits) + p.fxsum, sk.bad, s_mag[k] == 0);
+            const FxUnit un(sk.unit(p.fxbits) + (DYN ? s_sum[k] : esum), sk.bad, s_mag[k] == 0);
             for (int e = threadIdx.x; e <= n; e += blockDim.x) {
                 const fxc v = r[e * LD + k];
                 tile[k * a.ls + e] = fx_to_odd(v, un);
             }
         }
     } else if (l < live) {
-        const FxUnit un(sc.unit(p.fxbits) + p.fxsum, sc.bad, s_mag[l] == 0);
+        const FxUnit un(sc.unit(p.fxbits) + esum, sc.bad, s_mag[l] == 0);
         for (int e = g; e <= n; e += m) {
             const fxc v = r[e * LD + l];
             tile[l * a.ls + e * a.es] = fx_to_odd(v, un);

@@ -131,12 +131,13 @@ struct FftPlan {
     int nst;
     int radix[12];
 };
-// With its fixed-point runs (apply_fxg.cuh): K of each stage, bits of the inputs, and the sum of the K
-// by which the outputs' unit is coarser than the inputs'.  (The other engines' kernels take the plan
-// alone: with these fields in it they ran 2% slower.)
+// With its fixed-point runs (fxg.cuh): K of each stage, bits of the inputs, and the sum of the K by which
+// the outputs' unit is coarser than the inputs'; fxdyn: K follows the values instead.  (The other
+// engines' kernels take the plan alone: with these fields in it they ran 2% slower.)
 struct FxPlan : FftPlan {
     int fxk[12];
     int fxbits, fxsum;
+    bool fxdyn;
 };
 
 }  // namespace lsm

@@ -8,7 +8,7 @@
 // only products round, to one unit of the last place.  The results' unit is 2^-57 (L = 16) to 2^-53
 // (inverse transforms of L = 512) of the line's largest input; the first step, and half of the
 // 32-point DFT, work in units 4 to 16 times finer.  (FP64's own unit is 2^-53 of each value.)  Against
-// longdouble a line's rms error is 0.16 to 1.0 of that of the same plan in FP64, in the worst of six
+// longdouble a line's rms error is 0.2 to 1.0 of that of the same plan in FP64, in the worst of six
 // kinds of fields 0.88 on inverse lines at L = 512 (tests/test_fixed_point_lines.py).  Inputs and
 // outputs stay FP64 in memory.
 // Measured at 128^3, one system: FP64 apply 9.05 -> 2.13 ms (z pass 5.21 -> 0.93, y passes 1.05 -> 0.175
@@ -197,6 +197,10 @@ __device__ __forceinline__ fxc fx_cmul_quarter(fxc a, long long kr, long long ki
 __device__ __forceinline__ fxr fx_shift(fxr v, int sh) {
     if (sh > 0) return fx_r(((fx_ll(v) >> min(sh - 1, 62)) + 1) >> 1);
     return fx_r((long long)((unsigned long long)fx_ll(v) << min(-sh, 63)));
+}
+// high words of the components' moduli (less one for negative ones), or-ed
+__device__ __forceinline__ unsigned fx_hibits(fxc v) {
+    return (unsigned)((v.x.h ^ (v.x.h >> 31)) | (v.y.h ^ (v.y.h >> 31)));
 }
 // +-a +-b
 __device__ __forceinline__ fxr fx_pm(fxr a, bool pa, fxr b, bool pb) {

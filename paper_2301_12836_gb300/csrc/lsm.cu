@@ -6,7 +6,7 @@
 // runs in the kernels of apply.cu, green.cu and solver.cu.
 #include "lsm.h"
 #include "kernels.h"
-#include "fx.cuh"
+#include "fxg.cuh"
 #include "solver.cuh"
 
 #include <cmath>
@@ -145,41 +145,6 @@ lsm_status cuda_fail(lsm_t h, cudaError_t e, const char* where) {
         cudaError_t _e = (call);                             \
         if (_e != cudaSuccess) return cuda_fail(h, _e, #call); \
     } while (0)
-
-// Scaling of a plan's fixed-point stages: in log2 of the largest modulus, the first stage's outputs and
-// every later stage's stay below 61.9 with the smallest K in 1 .. 3 that does it (K = 1 doubles the
-// values before a product, which needs them below 60.9).
-void fixed_point_scaling(FxPlan& p) {
-    const double top = 61.9;
-    const double g0 = log2((double)p.radix[0]);
-    p.fxbits = (int)floor(top - 0.5 - g0);
-    double m = p.fxbits + 0.5 + g0;
-    p.fxk[0] = 0;
-    p.fxsum = 0;
-    for (int s = 1; s < p.nst; ++s) {
-        const double g = log2((double)p.radix[s]);
-        int k = (m <= top - 1.0 && m + g - 1.0 <= top) ? 1 : (m + g - 2.0 <= top ? 2 : 3);
-        p.fxk[s] = k;
-        p.fxsum += k;
-        m += g - k;
-    }
-}
-
-bool factor_plan(int L, FxPlan& p) {
-    p.L = L;
-    p.nst = 0;
-    int m = L;
-    const int rs[5] = {8, 4, 2, 3, 5};
-    for (int k = 0; k < 5; ++k) {
-        while (m % rs[k] == 0) {
-            if (p.nst >= 12) return false;
-            p.radix[p.nst++] = rs[k];
-            m /= rs[k];
-        }
-    }
-    if (m == 1) fixed_point_scaling(p);
-    return m == 1;
-}
 
 // exp(-2 pi i k / L), k < L, evaluated in long double and rounded once; fx2, fx3: as fixed-point words
 // times 2^-2 and 2^-3

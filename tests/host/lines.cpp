@@ -1,9 +1,10 @@
 // Single lines of the FP64 transforms' engines, thread by thread on the CPU: the fixed-point engine
-// (csrc/fx.cuh, fft4.cuh) and the same plan in FP64 against long double.
+// (csrc/fx.cuh, fft4.cuh, fxg.cuh) and the same plan in FP64 against long double.
 //   lines accuracy   per length, field and direction: rms relative errors of both engines
 //   lines range      per plan: range errors (sums or factors that leave their words) over lines at
 //                    the full scale, aligned with each frequency in turn
 #include "fft4.cuh"
+#include "fxg.cuh"
 
 #include <complex>
 #include <cstdio>
@@ -86,6 +87,46 @@ template <int A, int B> struct TwoStep : Plan {
     }
     void raw(int S, const fxc* in, int, const Tables& T) const override {
         any(S, in, T.fx[fx_twiddle_k(A * B)].data(), [](int, fxc) {});
+    }
+};
+
+// the runtime engine, one thread for a tile of one line
+struct Runtime : Plan {
+    FxPlan p;
+    explicit Runtime(int len) {
+        L = len;
+        factor_plan(len, p);
+    }
+    int scale_bits(int, int) const override { return p.fxbits; }
+    template <int S, bool DYN> fxc* run(std::vector<fxc>& a, std::vector<fxc>& b, const Tables& T, int& esum) const {
+        unsigned hi[3] = {0, 0, 0};
+        return fxg_fft<S, 1, DYN, 1>(a.data(), b.data(), p, FxTables{T.fx[2].data(), T.fx[3].data()}, 0, 0, 1, hi, 0, esum);
+    }
+    fxc* any(int S, std::vector<fxc>& a, std::vector<fxc>& b, const Tables& T, int& esum) const {
+        if (S < 0) return p.fxdyn ? run<-1, true>(a, b, T, esum) : run<-1, false>(a, b, T, esum);
+        return p.fxdyn ? run<1, true>(a, b, T, esum) : run<1, false>(a, b, T, esum);
+    }
+    void fixed(int S, const Line& in, int, Line& out, const Tables& T) const override {
+        unsigned mag = 0;
+        for (const double2& v : in) mag = max(mag, max(fx_mag(v.x), fx_mag(v.y)));
+        const FxScale sc(mag);
+        std::vector<fxc> q, b(L);
+        for (const double2& v : in) q.push_back(fx_from(v, sc, p.fxbits));
+        int esum;
+        const fxc* r = any(S, q, b, T, esum);
+        const FxUnit un(sc.unit(p.fxbits) + esum, sc.bad, mag == 0);
+        for (int k = 0; k < L; ++k) out[k] = un.odd ? fx_to_odd(r[k], un) : fx_to(r[k], un);
+    }
+    void fp64(int S, const Line& in, Line& out, const Tables& T) const override {
+        Line a = in, b(L);
+        const double2* r = S < 0 ? fft_smem<-1>(a.data(), b.data(), p, 1, 1, T.d.data(), 0, 1)
+                                 : fft_smem<1>(a.data(), b.data(), p, 1, 1, T.d.data(), 0, 1);
+        for (int k = 0; k < L; ++k) out[k] = r[k];
+    }
+    void raw(int S, const fxc* in, int, const Tables& T) const override {
+        std::vector<fxc> a(in, in + L), b(L);
+        int esum;
+        any(S, a, b, T, esum);
     }
 };
 
@@ -214,5 +255,10 @@ int main(int argc, char** argv) {
     go(TwoStep<8, 16>());
     go(TwoStep<16, 16>());
     go(TwoStep<16, 32>());
+    // the runtime engine: short plans, every radix last, the longest static plans, dynamic plans of
+    // every first and last radix
+    for (int L : {12, 18, 30, 48, 64, 90, 100, 120, 128, 192, 200, 256, 144, 150, 162, 180, 240, 250, 270, 288, 300, 320, 360, 384, 400,
+                  432, 450, 480, 486, 500, 512})
+        go(Runtime(L));
     return 0;
 }

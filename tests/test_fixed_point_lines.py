@@ -38,12 +38,12 @@ def lines(tmp_path_factory):
 
 def test_accuracy_no_worse_than_fp64(lines):
     rows = lines("accuracy")
-    assert len(rows) >= 6 * 12
+    assert len(rows) >= 37 * 12
     worse = [r for r in rows if float(r[3]) > float(r[4])]
     assert not worse, worse
 
 
 def test_full_scale_lines_stay_in_range(lines):
     rows = lines("range")
-    assert len(rows) >= 6 * 4
+    assert len(rows) >= 37 * 4
     assert all(int(r[4]) == 0 for r in rows), rows

@@ -1,5 +1,5 @@
 """The FP64 operator's fixed-point transforms on 512-point lines (sides of 256), along each axis, and its
-accuracy on a side of every two-step length.
+accuracy on a side of every two-step length and on long lines of the runtime engine.
 
 Accuracy, per displacement component, forward and adjoint: the distance from the longdouble value is
 at most twice that of a NumPy evaluation of the same formulas in FP64 (the two differ in the order of
@@ -18,6 +18,7 @@ from gpu_helpers import dev, field, handle, host
 pytestmark = pytest.mark.gpu
 
 LONG = [(256, 5, 6), (5, 256, 6), (6, 5, 256)]
+GENERIC = [(81, 5, 6), (5, 125, 6), (6, 5, 144), (180, 5, 4), (5, 225, 4), (4, 5, 250), (243, 4, 5), (5, 4, 240)]
 SIDES = [(8, 16, 32), (64, 9, 8), (8, 128, 9)] + LONG
 
 
@@ -34,7 +35,7 @@ def _setup(n, seed):
     return med, w
 
 
-@pytest.mark.parametrize("n", SIDES)
+@pytest.mark.parametrize("n", SIDES + GENERIC)
 def test_components_against_longdouble(n):
     med, w = _setup(n, 51)
     h = handle(med, w)
