@@ -401,9 +401,12 @@ __global__ void __launch_bounds__(3 * TX * FourStep<A LSM_COMMA B>::TPL, 2) k4_f
         }
     double2* __restrict__ dst = pick<double2>(S, dst_sel) + (size_t)cl * out_count * plane;
     auto st_g = [&](int, int k, fxc r, auto odd) {
-        // the shift above rounded L inputs down, half a unit of the first step each on average:
-        // a sum that lands on output 0 alone
-        if (k == 0) r = cadd(r, fxc{fxr{L >> (fx_prescale(L) + 1), 0}, fxr{L >> (fx_prescale(L) + 1), 0}});
+        // the shift above rounded L inputs down, half a unit of the first step each on average: a sum
+        // that lands on output 0 alone (a component that is zero in the whole column stays zero)
+        if (k == 0) {
+            constexpr unsigned half = L >> (fx_prescale(L) + 1);
+            r = fxc{fx_add(r.x, fxr{r.x.l | (unsigned)r.x.h ? half : 0u, 0}), fx_add(r.y, fxr{r.y.l | (unsigned)r.y.h ? half : 0u, 0})};
+        }
         const int eo = k - out_off;
         if (xin && eo >= 0 && eo < out_count) dst[(unsigned)eo * plane + col] = odd() ? fx_to_odd(r, un) : fx_to(r, un);
     };

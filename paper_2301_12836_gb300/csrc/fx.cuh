@@ -320,7 +320,6 @@ struct FxUnit {
         odd = nan || zero || E < -1021 || E > 960;
     }
 };
-// a zero comes out as +-2^(E - 2), a quarter of the unit
 __device__ __forceinline__ double fx_to(fxr v, const FxUnit& u) {
     const int sg = v.h >> 31;
     const fxr m = fx_sub(fxr{v.l ^ (unsigned)sg, v.h ^ sg}, fxr{(unsigned)sg, sg});   // < 2^63
@@ -328,7 +327,7 @@ __device__ __forceinline__ double fx_to(fxr v, const FxUnit& u) {
     const int lz = __clz(small ? (int)m.l : m.h) + (small ? 31 : -1);   // one less than the leading zeros: leading bit to 62
     const unsigned long long n = ((unsigned long long)fx_ll(m) << lz) + 0x1ff;
     const unsigned h = (unsigned)(n >> 42) + ((unsigned)(u.e - 1 - lz) << 20);   // a carry goes into the exponent
-    return __hiloint2double((int)(h | ((unsigned)sg & 0x80000000u)), (int)(unsigned)(n >> 10));
+    return __hiloint2double(small && m.l == 0 ? 0 : (int)(h | ((unsigned)sg & 0x80000000u)), (int)(unsigned)(n >> 10));
 }
 __device__ __forceinline__ double2 fx_to(fxc v, const FxUnit& u) { return make_double2(fx_to(v.x, u), fx_to(v.y, u)); }
 __device__ __forceinline__ double fx_to_odd(fxr v, const FxUnit& u) {

@@ -3,12 +3,14 @@
 //   lines accuracy   per length, field and direction: rms relative errors of both engines
 //   lines range      per plan: range errors (sums or factors that leave their words) over lines at
 //                    the full scale, aligned with each frequency in turn
+//   lines zeros      per plan and direction: outputs that cancel exactly but come out nonzero
 #include "fft4.cuh"
 #include "fxg.cuh"
 
 #include <complex>
 #include <cstdio>
 #include <random>
+#include <string>
 #include <vector>
 
 using namespace lsm;
@@ -246,9 +248,27 @@ static void range(const Plan& p) {
     }
 }
 
+// Two equal elements half a line apart: every odd output is x - x
+static void zeros(const Plan& p) {
+    const int L = p.L;
+    const Tables T(L);
+    for (int S = -1; S <= 1; S += 2) {
+        Line in(L, double2{0, 0}), out(L, double2{0, 0});
+        in[0] = in[L / 2] = double2{0.3, -1.7};
+        p.fixed(S, in, S < 0 ? L / 2 + 1 : L, out, T);
+        int bad = 0;
+        for (int k = 1; k <= L / 2; k += 2) bad += out[k].x != 0.0 || out[k].y != 0.0;
+        std::printf("%d %d %d\n", L, S, bad);
+    }
+}
+
 int main(int argc, char** argv) {
-    const bool acc = argc > 1 && std::string(argv[1]) == "accuracy";
-    auto go = [&](const Plan& p) { acc ? accuracy(p) : range(p); };
+    const std::string what = argc > 1 ? argv[1] : "";
+    auto go = [&](const Plan& p) {
+        if (what == "accuracy") accuracy(p);
+        else if (what == "range") range(p);
+        else zeros(p);
+    };
     go(TwoStep<4, 4>());
     go(TwoStep<4, 8>());
     go(TwoStep<8, 8>());

@@ -6,6 +6,7 @@
   inverse lines of their spectra times a Green spectrum, at 10 and 25 nodes per wave.
 * Range: no sum and no factor leaves its words on lines at the full scale, aligned with each
   frequency in turn so that the whole headroom is used.
+* Outputs that cancel exactly are zero.
 """
 import os
 import platform
@@ -22,7 +23,7 @@ pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="needs a hos
 
 @pytest.fixture(scope="module")
 def lines(tmp_path_factory):
-    """Rows (as lists of words) of `lines accuracy` or `lines range`."""
+    """Rows (as lists of words) of `lines <what>`."""
     exe = str(tmp_path_factory.mktemp("lines") / "lines")
     fma = []   # the FP64 yardstick uses fused multiply-adds, as the GPU does
     if platform.machine() == "x86_64" and "fma" in open("/proc/cpuinfo").read().split():
@@ -47,3 +48,9 @@ def test_full_scale_lines_stay_in_range(lines):
     rows = lines("range")
     assert len(rows) >= 37 * 4
     assert all(int(r[4]) == 0 for r in rows), rows
+
+
+def test_exact_cancellations_are_zero(lines):
+    rows = lines("zeros")
+    assert len(rows) >= 37 * 2
+    assert all(int(r[2]) == 0 for r in rows), rows
