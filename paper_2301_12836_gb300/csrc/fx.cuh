@@ -195,7 +195,7 @@ __device__ __forceinline__ fxc fx_cmul_quarter(fxc a, long long kr, long long ki
 }
 // v 2^-sh, rounded to nearest, for sh of either sign; 64 or more shifts any value out
 __device__ __forceinline__ fxr fx_shift(fxr v, int sh) {
-    if (sh > 0) return fx_r(((fx_ll(v) >> min(sh - 1, 62)) + 1) >> 1);
+    if (sh > 0) return fx_r(((fx_ll(v) >> min(sh - 1, 63)) + 1) >> 1);
     return fx_r((long long)((unsigned long long)fx_ll(v) << min(-sh, 63)));
 }
 // high words of the components' moduli (less one for negative ones), or-ed
@@ -308,8 +308,10 @@ __device__ __forceinline__ fxc fx_from(double2 v, const FxScale& s, int bits) {
     return fxc{fx_from(v.x, s, bits), fx_from(v.y, s, bits)};
 }
 
-// v 2^E rounded to FP64 (to nearest, ties towards zero); results below the normal range give zero,
-// results above it infinity
+// v 2^E rounded to FP64 (to nearest), with gradual underflow; results above the range are infinite.  Ties
+// go towards zero: either constant costs one addition where ties to even take two instructions more,
+// and the rms error of a line is the same under the three rules (mean ratio over 444 sets of lines
+// 0.999, 0.999).
 struct FxUnit {
     int e;       // E + 1085: one below the biased exponent of a value with no leading zeros
     bool odd;    // some v gives no normal number, or the line is bad or zero: fx_to_odd
@@ -337,7 +339,8 @@ __device__ __forceinline__ double fx_to_odd(fxr v, const FxUnit& u) {
     if ((m.h | (int)m.l) == 0) return 0.0;
     const int be = u.e + 1 - (m.h ? __clz(m.h) : 32 + __clz((int)m.l));   // biased exponent
     if (be >= 1 && be <= 2046) return fx_to(v, u);
-    return __hiloint2double((be < 1 ? 0 : 0x7ff00000) | (sg & (int)0x80000000), 0);
+    const fxr q = be < 1 ? fx_shift(m, 11 - u.e) : fxr{0u, 0x7ff00000};   // below the normal range: in units of 2^-1074
+    return __hiloint2double(q.h | (sg & (int)0x80000000), (int)q.l);
 }
 __device__ __forceinline__ double2 fx_to_odd(fxc v, const FxUnit& u) { return make_double2(fx_to_odd(v.x, u), fx_to_odd(v.y, u)); }
 

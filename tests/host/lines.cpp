@@ -4,6 +4,7 @@
 //   lines range      per plan: range errors (sums or factors that leave their words) over lines at
 //                    the full scale, aligned with each frequency in turn
 //   lines zeros      per plan and direction: outputs that cancel exactly but come out nonzero
+//   lines convert    conversions to FP64 that are not the nearest value (either one at a tie)
 #include "fft4.cuh"
 #include "fxg.cuh"
 
@@ -262,8 +263,28 @@ static void zeros(const Plan& p) {
     }
 }
 
+static void convert() {
+    long bad = 0, subnormal = 0;
+    for (int i = 0; i < 400000; ++i) {
+        const long long v = (long long)((unsigned long long)((long long)(rng() >> 1) >> (i % 63)) << (i / 63 % 3));
+        const int E = -1140 + (int)(rng() % 2110);
+        if (v < 0) continue;
+        const long double exact = ldexpl((long double)(i & 1 ? -v : v), E);
+        const FxUnit un(E, false, false);
+        const double got = un.odd ? fx_to_odd(fx_r(i & 1 ? -v : v), un) : fx_to(fx_r(i & 1 ? -v : v), un);
+        const double near = (double)exact;
+        subnormal += near != 0.0 && std::fabs(near) < 2.2250738585072014e-308;
+        if (std::isinf(near) ? got != near : fabsl(got - exact) != fabsl(near - exact)) ++bad;
+    }
+    std::printf("%ld %ld\n", bad, subnormal);
+}
+
 int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
+    if (what == "convert") {
+        convert();
+        return 0;
+    }
     auto go = [&](const Plan& p) {
         if (what == "accuracy") accuracy(p);
         else if (what == "range") range(p);

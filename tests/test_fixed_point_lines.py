@@ -6,7 +6,8 @@
   inverse lines of their spectra times a Green spectrum, at 10 and 25 nodes per wave.
 * Range: no sum and no factor leaves its words on lines at the full scale, aligned with each
   frequency in turn so that the whole headroom is used.
-* Outputs that cancel exactly are zero.
+* Outputs that cancel exactly are zero, and conversions give the nearest FP64 value down to the
+  smallest subnormal.
 """
 import os
 import platform
@@ -54,3 +55,9 @@ def test_exact_cancellations_are_zero(lines):
     rows = lines("zeros")
     assert len(rows) >= 37 * 2
     assert all(int(r[2]) == 0 for r in rows), rows
+
+
+def test_conversion_to_fp64_is_nearest(lines):
+    (bad, subnormal), = lines("convert")
+    assert int(subnormal) > 5000
+    assert int(bad) == 0

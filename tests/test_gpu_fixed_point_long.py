@@ -77,3 +77,18 @@ def test_long_lines_zero_infinite_and_nan(n):
         v = u.copy()
         v[2, n[2] // 2, n[1] // 3, n[0] // 3] = bad
         assert np.all(np.isnan(_apply(h, v)))
+
+
+def test_subnormal_results():
+    """A field of 2^-1035: the displacements, and the transforms' intermediates that stand for them, lie
+    below the normal range, where a value keeps 2^-1074.  Relative to u that is 2^-39; the strain's
+    1 / 2h, the spectrum's 1 / P and the sums over a line lose at most 12 bits more.  (The adjoint's
+    first intermediate is about 2^-30 u, the kernel before the contrast: there FP64 itself keeps 9 bits.)"""
+    n = (8, 16, 32)
+    med, w = _setup(n, 54)
+    h = handle(med, w)
+    u = field(med.shape, 24)
+    s = 2.0 ** -1035
+    scattered = u - _apply(h, u)
+    got = (u * s - _apply(h, u * s)) * 2.0 ** 600 * 2.0 ** 435   # 1 / s is out of range
+    assert np.linalg.norm(got - scattered) < 2.0 ** -27 * np.linalg.norm(scattered)
