@@ -115,6 +115,16 @@ template <int N> __device__ __forceinline__ void cp_async_wait_group() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// Element i of a fixed white field, uniform in (-1, 1) and never zero (SplitMix64's output function,
+// Steele, Lea and Flood 2014).
+__host__ __device__ __forceinline__ double white(unsigned long long i) {
+    unsigned long long z = (i + 1) * 0x9e3779b97f4a7c15ULL;
+    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
+    z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
+    z ^= z >> 31;
+    return ((double)(long long)(z >> 32) - 2147483647.5) / 2147483648.0;
+}
+
 // Grid geometry of one medium.  Model nodes n_a; padded periodic length L_a = 2 n_a;
 // extended contrast-source nodes e_a = n_a + 2 (nodes -1 .. n_a).
 struct Dims {

@@ -427,6 +427,11 @@ __global__ void k_f2d_c(const float2* __restrict__ in, double2* __restrict__ out
         out[i] = make_double2((double)in[i].x, (double)in[i].y);
 }
 
+template <typename T> __global__ void k_white(T* __restrict__ out, long long n) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = (T)white((unsigned long long)i);
+}
+
 // double -> double-float: hi = fl32(v), lo = fl32(v - hi); |lo| <= ulp(hi) / 2
 __global__ void k_d2df(const double* __restrict__ in, dfloat* __restrict__ out, long long n) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -439,6 +444,14 @@ __global__ void k_df2d(double* buf, long long n) {
         buf[i] = (double)v.x + (double)v.y;
     }
 }
+
+template <typename T> cudaError_t launch_white(T* out, long long n, cudaStream_t st, long long* nl) {
+    k_white<T><<<gsz(n), 256, 0, st>>>(out, n);
+    if (nl) *nl += 1;
+    return cudaGetLastError();
+}
+template cudaError_t launch_white<float>(float*, long long, cudaStream_t, long long*);
+template cudaError_t launch_white<double>(double*, long long, cudaStream_t, long long*);
 
 cudaError_t launch_d2df(const double* in, dfloat* out, long long n, cudaStream_t st, long long* nl) {
     k_d2df<<<gsz(n), 256, 0, st>>>(in, out, n);

@@ -122,6 +122,9 @@ cudaError_t launch_octant_fft(const Dims& d, const Plans& pl64, double2* buf, cu
 cudaError_t launch_spectrum_forms(const double2* g, double scale, long long NO, int4* gx, int* ge, float2* g32, dfcplx* gdf,
                                   cudaStream_t st, long long* nlaunch);
 
+// n values of the white field of common.cuh
+template <typename T> cudaError_t launch_white(T* out, long long n, cudaStream_t st, long long* nlaunch);
+
 // Precision converters.  d2df: n reals to double-float pairs; df2d_inplace: n double-float pairs
 // to doubles in the same memory (8 bytes each).
 cudaError_t launch_d2df(const double* in, dfloat* out, long long n, cudaStream_t st, long long* nlaunch);
