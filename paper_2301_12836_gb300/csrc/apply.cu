@@ -1596,15 +1596,19 @@ static void launch_rows_fxg(const Dims& d, const ApplySys<double>* sys, int nsys
 }
 
 // x FFT of nrows contiguous rows: in_count elements at in_off of each line (forward: the rest zero),
-// outputs out_off .. out_off + out_count - 1: src_sel -> dst_sel
+// outputs out_off .. out_off + out_count - 1: src_sel -> dst_sel.  The FP32 and double-float two-step
+// kernels are forward ones of whole lines from offset 0 (the operator's); any other form of theirs runs
+// on the generic engine.
 template <typename T, int DIR>
 static void launch_xrows(const Dims& d, const ApplySys<T>* sys, int nsys, const Plans& pl, int src_sel, int dst_sel,
                          long long nrows, int in_count, int in_off, int out_count, int out_off, cudaStream_t st, int v = 0) {
     typedef typename cplx_of<T>::type C;
     if (!fourstep_prunable(d.Lx, DIR < 0 ? in_off + in_count : 0, DIR > 0 ? out_off + out_count : 0)) v = 1;
+    constexpr bool FX = std::is_same<T, double>::value;
+    if (!FX && (DIR > 0 || in_off != 0 || out_off != 0 || out_count != d.Lx)) v = 1;
     with_engine<std::is_same<T, dfloat>::value>(d.Lx, [&](auto eng) {
         using F = decltype(eng);
-        if constexpr (std::is_same<T, double>::value) {
+        if constexpr (FX) {
             if constexpr (F::INPLACE) {
                 constexpr int A = F::A_, B = F::B_, LPB = 128 / F::TPL;
                 const size_t sm = (size_t)LPB * B * (A + 1) * sizeof(fxc);
@@ -1615,11 +1619,11 @@ static void launch_xrows(const Dims& d, const ApplySys<T>* sys, int nsys, const 
             } else {
                 launch_rows_fxg<DIR, false>(d, sys, nsys, pl, src_sel, dst_sel, nrows, in_count, in_off, out_count, out_off, st, v);
             }
-        } else if constexpr (F::INPLACE && F::A_ == F::B_) {
+        } else if constexpr (F::INPLACE && DIR < 0 && F::A_ == F::B_) {
             constexpr int A = F::A_, LPB = sizeof(T) == 4 ? 16 : 8;
             k4_rows_w<T, A, LPB><<<dim3(cdiv(nrows, LPB), nsys), LPB * A, 0, st>>>((const C*)pl.twx, sys, src_sel, dst_sel,
                                                                                    nrows, in_count);
-        } else if constexpr (F::INPLACE) {
+        } else if constexpr (F::INPLACE && DIR < 0) {
             constexpr int A = F::A_, B = F::B_, LPB = RowsW2<A, B>::LPB;   // FP32 only: double-float has no A != B engine
             k4_rows_w2<A, B><<<dim3(cdiv(nrows, LPB), nsys), 128, 0, st>>>((const C*)pl.twx, sys, src_sel, dst_sel, nrows, in_count);
         } else {
@@ -2020,7 +2024,7 @@ template <typename T>
 static void launch_adjoint_conv(const Medium& m, const Plans& pl, const ApplySys<T>* sys, int nsys, cudaStream_t st) {
     const Dims& d = m.d;
     // 1. w placed at x positions 1..nx, forward x FFT: u [3][nz][ny][nx] -> w1 [3][nz][ny][Lx]
-    launch_xrows<T, -1>(d, sys, nsys, pl, 0, 2, 3LL * d.nz * d.ny, d.nx, 1, d.Lx, 0, st, std::is_same<T, double>::value ? 0 : 1);
+    launch_xrows<T, -1>(d, sys, nsys, pl, 0, 2, 3LL * d.nz * d.ny, d.nx, 1, d.Lx, 0, st);
     // 2. forward y FFT, input at 1..ny: w1 [3][nz][ny][Lx] -> w2 [3][nz][Ly][Lx]
     launch_ypass<T, -1>(d, sys, nsys, pl, d.nz, d.ny, 1, d.Ly, 0, 2, 3, st);
     // 3. z: input at 1..nz, conj(G-hat), output extended 0..ez-1: w2 -> w1 [3][ez][Ly][Lx]
@@ -2028,7 +2032,7 @@ static void launch_adjoint_conv(const Medium& m, const Plans& pl, const ApplySys
     // 4. inverse y FFT, keep 0..ey-1: w1 [3][ez][Ly][Lx] -> w2 [3][ez][ey][Lx]
     launch_ypass<T, 1>(d, sys, nsys, pl, d.ez, d.Ly, 0, d.ey, 0, 2, 3, st);
     // 5. inverse x FFT, keep 0..ex-1: w2 [3][ez][ey][Lx] -> w1 [3][ez][ey][ex]
-    launch_xrows<T, 1>(d, sys, nsys, pl, 3, 2, 3LL * d.ez * d.ey, d.Lx, 0, d.ex, 0, st, std::is_same<T, double>::value ? 0 : 1);
+    launch_xrows<T, 1>(d, sys, nsys, pl, 3, 2, 3LL * d.ez * d.ey, d.Lx, 0, d.ex, 0, st);
 }
 
 template <typename T>
