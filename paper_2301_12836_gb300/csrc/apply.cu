@@ -31,37 +31,19 @@ namespace lsm {
 static constexpr int NTH = 256;
 
 // FFT engines.  GenericFFT: runtime mixed-radix Stockham plan, ping-pong buffers, any block size.
-// FourStepFFT<A, B>: compile-time L = A * B, in place, exactly NL * TPL threads per block.
-// Launch bounds of the FFT kernels.  Four-step tiles have at most 384 threads (FP32) or 192
-// (FP64); asking for two resident FP32 blocks keeps those kernels at <= 85 registers, while the
-// FP64 ones keep their 16-point DFTs in up to 255 registers without spilling.
-template <typename T, bool INPLACE> struct FftBounds {
-    static constexpr int threads = INPLACE ? (sizeof(T) == 8 ? 192 : 384) : 512;
-    static constexpr int blocks = (INPLACE && sizeof(T) == 4) ? 2 : 1;
-};
-#define LSM_COMMA ,
-#define LSM_FFT_BOUND(T, F) __launch_bounds__(FftBounds<T LSM_COMMA F::INPLACE>::threads, FftBounds<T LSM_COMMA F::INPLACE>::blocks)
-
+// FourStepFFT<A, B>: compile-time L = A * B; its kernels run NL * TPL threads.
 struct GenericFFT {
     static constexpr bool INPLACE = false;
     static constexpr int TPL = 0;
     static constexpr int A_ = 0, B_ = 0;
-    template <int S, typename C>
-    static __device__ __forceinline__ C* run(C* a, C* b, const FftPlan& p, int NL, int LD, const C* __restrict__ tw) {
-        return fft_smem<S>(a, b, p, NL, LD, tw, threadIdx.x, blockDim.x);
-    }
 };
 template <int A, int B>
 struct FourStepFFT {
     static constexpr int A_ = A, B_ = B;
     static constexpr bool INPLACE = true;
     static constexpr int TPL = FourStep<A, B>::TPL;
-    template <int S, typename C>
-    static __device__ __forceinline__ C* run(C* a, C*, const FftPlan&, int NL, int LD, const C* __restrict__ tw) {
-        fft4_smem<A, B, S>(a, NL, LD, tw, threadIdx.x);
-        return a;
-    }
 };
+#define LSM_COMMA ,
 
 // Voigt index (order 11, 22, 33, 23, 13, 12) of the tensor pair (j, k).
 __device__ __forceinline__ int t2v(int j, int k) { return (j == k) ? j : (6 - j - k); }
@@ -293,7 +275,7 @@ __device__ __forceinline__ C* pick(const ApplySys<typename real_of<C>::type>& S,
     }
 }
 
-template <int DIR, class F, typename C>
+template <int DIR, typename C>
 __device__ __forceinline__ void strided_tile(const C* src, C* dst, const FftPlan& p, const C* __restrict__ tw,
                                              const StridedArgs& a, int x0, C* sa, C* sb) {
     const int L = p.L, TX = a.TX;
@@ -307,7 +289,7 @@ __device__ __forceinline__ void strided_tile(const C* src, C* dst, const FftPlan
         sa[i] = v;
     }
     __syncthreads();
-    C* r = F::template run<DIR>(sa, sb, p, TX, TX, tw);
+    C* r = fft_smem<DIR>(sa, sb, p, TX, TX, tw, threadIdx.x, blockDim.x);
     for (int i = threadIdx.x; i < a.out_count * TX; i += blockDim.x) {
         const int l = i % TX;
         const int eo = i / TX;
@@ -316,8 +298,8 @@ __device__ __forceinline__ void strided_tile(const C* src, C* dst, const FftPlan
     }
 }
 
-template <typename T, int DIR, class F>
-__global__ void LSM_FFT_BOUND(T, F) k_strided(FftPlan p, const typename cplx_of<T>::type* __restrict__ tw,
+template <typename T, int DIR>
+__global__ void __launch_bounds__(512) k_strided(FftPlan p, const typename cplx_of<T>::type* __restrict__ tw,
                                                  StridedArgs a, const ApplySys<T>* __restrict__ sys) {
     typedef typename cplx_of<T>::type C;
     extern __shared__ unsigned char smem_raw[];
@@ -326,10 +308,10 @@ __global__ void LSM_FFT_BOUND(T, F) k_strided(FftPlan p, const typename cplx_of<
     const ApplySys<T> S = sys[s];
     if (S.run && !*S.run) return;
     C* sa = reinterpret_cast<C*>(smem_raw);
-    C* sb = F::INPLACE ? sa : sa + (size_t)p.L * a.TX;
+    C* sb = sa + (size_t)p.L * a.TX;
     const C* src = pick<C>(S, a.src_sel) + c * a.src_os2 + blockIdx.y * a.src_os1;
     C* dst = pick<C>(S, a.dst_sel) + c * a.dst_os2 + blockIdx.y * a.dst_os1;
-    strided_tile<DIR, F>(src, dst, p, tw, a, blockIdx.x * a.TX, sa, sb);
+    strided_tile<DIR>(src, dst, p, tw, a, blockIdx.x * a.TX, sa, sb);
 }
 
 // raw-pointer variant for the Green spectrum setup (in place allowed: each CTA owns its tile)
@@ -343,7 +325,7 @@ __global__ void __launch_bounds__(NTH) k_strided_raw(FftPlan p, const typename c
     C* sb = sa + (size_t)p.L * a.TX;
     const C* src = src0 + blockIdx.z * a.src_os2 + blockIdx.y * a.src_os1;
     C* dst = dst0 + blockIdx.z * a.dst_os2 + blockIdx.y * a.dst_os1;
-    strided_tile<DIR, GenericFFT>(src, dst, p, tw, a, blockIdx.x * a.TX, sa, sb);
+    strided_tile<DIR>(src, dst, p, tw, a, blockIdx.x * a.TX, sa, sb);
 }
 
 }  // namespace lsm
@@ -794,8 +776,8 @@ __global__ void __launch_bounds__(4 * TX * A, A == 16 ? 2 : 4) k4z_pair2(
 // adjoint), inverse z FFT.  CTA: TX lines along x at one ky, all three components.
 // src [3][in_count][Ly][Lx] (sel), dst [3][out_count][Ly][Lx] (sel)
 // ---------------------------------------------------------------------------------------------
-template <typename T, bool CONJ, class F>
-__global__ void LSM_FFT_BOUND(T, F) k_fftz_green(Dims d, FftPlan pz, const typename cplx_of<T>::type* __restrict__ tw,
+template <typename T, bool CONJ>
+__global__ void __launch_bounds__(512) k_fftz_green(Dims d, FftPlan pz, const typename cplx_of<T>::type* __restrict__ tw,
                                                     const ApplySys<T>* __restrict__ sys, int TX, int in_count, int in_off,
                                                     int out_count, int out_off, int src_sel, int dst_sel) {
     typedef typename cplx_of<T>::type C;
@@ -804,7 +786,7 @@ __global__ void LSM_FFT_BOUND(T, F) k_fftz_green(Dims d, FftPlan pz, const typen
     if (S.run && !*S.run) return;
     const int L = d.Lz, NL = 3 * TX;
     C* sa = reinterpret_cast<C*>(smem_raw);
-    C* sb = F::INPLACE ? sa : sa + (size_t)L * NL;
+    C* sb = sa + (size_t)L * NL;
     const int ky = blockIdx.y;
     const int x0 = blockIdx.x * TX;
     const long long plane = (long long)d.Ly * d.Lx;
@@ -823,7 +805,7 @@ __global__ void LSM_FFT_BOUND(T, F) k_fftz_green(Dims d, FftPlan pz, const typen
         sa[e * NL + c * TX + lx] = v;
     }
     __syncthreads();
-    C* r = F::template run<-1>(sa, sb, pz, NL, NL, tw);
+    C* r = fft_smem<-1>(sa, sb, pz, NL, NL, tw, threadIdx.x, blockDim.x);
     C* o = (r == sa) ? sb : sa;
     for (int i = threadIdx.x; i < L * TX; i += blockDim.x) {
         const int lx = i % TX;
@@ -839,7 +821,7 @@ __global__ void LSM_FFT_BOUND(T, F) k_fftz_green(Dims d, FftPlan pz, const typen
         row[2 * TX] = cadd(cadd(cmul(G[4], q0), cmul(G[3], q1)), cmul(G[2], q2));
     }
     __syncthreads();
-    C* r2 = F::template run<1>(r, o, pz, NL, NL, tw);
+    C* r2 = fft_smem<1>(r, o, pz, NL, NL, tw, threadIdx.x, blockDim.x);
     for (int i = threadIdx.x; i < out_count * NL; i += blockDim.x) {
         const int lx = i % TX;
         const int rest = i / TX;
@@ -853,8 +835,8 @@ __global__ void LSM_FFT_BOUND(T, F) k_fftz_green(Dims d, FftPlan pz, const typen
 // ---------------------------------------------------------------------------------------------
 // inverse FFT along x + crop + Au = u - u_s.  CTA: B rows y at one z, 3 comps.  src w1 [3][nz][ny][Lx]
 // ---------------------------------------------------------------------------------------------
-template <typename T, class F>
-__global__ void LSM_FFT_BOUND(T, F) k_fftx_out(Dims d, const ApplySys<T>* __restrict__ sys, FftPlan px,
+template <typename T>
+__global__ void __launch_bounds__(512) k_fftx_out(Dims d, const ApplySys<T>* __restrict__ sys, FftPlan px,
                                                   const typename cplx_of<T>::type* __restrict__ tw, int B, int xoff) {
     typedef typename cplx_of<T>::type C;
     extern __shared__ unsigned char smem_raw[];
@@ -862,7 +844,7 @@ __global__ void LSM_FFT_BOUND(T, F) k_fftx_out(Dims d, const ApplySys<T>* __rest
     if (S.run && !*S.run) return;
     const int NL = 3 * B, LD = NL + 1, L = d.Lx;
     C* sa = reinterpret_cast<C*>(smem_raw);
-    C* sb = F::INPLACE ? sa : sa + (size_t)L * LD;
+    C* sb = sa + (size_t)L * LD;
     const int z = blockIdx.y;
     const int y0 = blockIdx.x * B;
     const C* __restrict__ src = S.w2;
@@ -876,7 +858,7 @@ __global__ void LSM_FFT_BOUND(T, F) k_fftx_out(Dims d, const ApplySys<T>* __rest
         sa[kx * LD + l] = v;
     }
     __syncthreads();
-    C* r = F::template run<1>(sa, sb, px, NL, LD, tw);
+    C* r = fft_smem<1>(sa, sb, px, NL, LD, tw, threadIdx.x, blockDim.x);
     for (int i = threadIdx.x; i < NL * d.nx; i += blockDim.x) {
         const int x = i % d.nx;
         const int l = i / d.nx;
@@ -954,8 +936,7 @@ __global__ void __launch_bounds__(NTH, sizeof(T) == 4 ? 6 : 1) k_divq(Dims d, co
 // elements), the transpose between the steps goes through a shared-memory tile private to the
 // line (row stride A + 1: conflict-free both ways) ordered by __syncwarp, and step 2 leaves
 // X[k1 + A k2] in registers for a coalesced store.  No block barrier and one shared-memory round
-// trip per element (a tile-transposing kernel makes three).  The arithmetic is that of fft4_smem,
-// operation for operation.
+// trip per element (a tile-transposing kernel makes three).
 template <int A, typename C>
 __device__ __forceinline__ void rows_w_exchange(C (&v)[A], C* tl, int q) {
 #pragma unroll
@@ -1516,19 +1497,11 @@ static void with_engine(int L, Fn&& fn, int v = 0) {
 }
 
 // tile of B rows x 3 components for the contiguous x passes
-template <typename T, class F>
-static void rows_cfg(int L, int& B, int& threads, size_t& sm, int shrink = 0) {
-    typedef typename cplx_of<T>::type C;
-    if constexpr (F::INPLACE) {
-        B = sizeof(T) == 4 ? 8 : 4;
-        threads = 3 * B * F::TPL;
-        sm = (size_t)L * (3 * B + 1) * sizeof(C);
-    } else {
-        B = rows_per_tile<T>(L) >> shrink;
-        if (B < 1) B = 1;
-        threads = NTH;
-        sm = 2 * (size_t)L * (3 * B + 1) * sizeof(C);
-    }
+template <typename T>
+static void rows_cfg(int L, int& B, size_t& sm, int shrink) {
+    B = rows_per_tile<T>(L) >> shrink;
+    if (B < 1) B = 1;
+    sm = 2 * (size_t)L * (3 * B + 1) * sizeof(typename cplx_of<T>::type);
 }
 // tile of TX consecutive lines x ncomp components for the strided passes
 template <typename T, class F>
@@ -1685,11 +1658,11 @@ static void launch_fftx_out(const Dims& d, const ApplySys<T>* sys, int nsys, con
             constexpr int A = F::A_, B = F::B_, LPB = RowsW2<A, B>::LPB;
             k4_xout_w2<A, B><<<dim3(cdiv(3LL * d.nz * d.ny, LPB), nsys), 128, 0, st>>>(d, sys, (const C*)pl.twx, xoff);
         } else {
-            int B, th;
+            int B;
             size_t sm;
-            rows_cfg<T, F>(d.Lx, B, th, sm, v == 2);
-            smem_attr((const void*)k_fftx_out<T, F>, sm);
-            k_fftx_out<T, F><<<dim3(cdiv(d.ny, B), d.nz, nsys), th, sm, st>>>(d, sys, pl.px, (const C*)pl.twx, B, xoff);
+            rows_cfg<T>(d.Lx, B, sm, v == 2);
+            smem_attr((const void*)k_fftx_out<T>, sm);
+            k_fftx_out<T><<<dim3(cdiv(d.ny, B), d.nz, nsys), NTH, sm, st>>>(d, sys, pl.px, (const C*)pl.twx, B, xoff);
         }
     }, v);
 }
@@ -1730,8 +1703,8 @@ static void launch_strided(int L, const FxPlan& p, const void* tw, const Plans& 
                 smem_attr((const void*)k4_strided<T, DIR, A, B, TXC>, sm);
                 k4_strided<T, DIR, A, B, TXC><<<dim3(cdiv(a.nlines, a.TX), outer, a.ncomp * nsys), th, sm, st>>>((const C*)tw, a, sys);
             } else {
-                smem_attr((const void*)k_strided<T, DIR, F>, sm);
-                k_strided<T, DIR, F><<<dim3(cdiv(a.nlines, a.TX), outer, a.ncomp * nsys), th, sm, st>>>(p, (const C*)tw, a, sys);
+                smem_attr((const void*)k_strided<T, DIR>, sm);
+                k_strided<T, DIR><<<dim3(cdiv(a.nlines, a.TX), outer, a.ncomp * nsys), th, sm, st>>>(p, (const C*)tw, a, sys);
             }
         }
     }, v);
@@ -1834,8 +1807,8 @@ static void launch_zpass(const Dims& d, const ApplySys<T>* sys, int nsys, const 
             k4_fftz_green<T, CONJ, A, B, TXC><<<dim3(cdiv(d.Lx, TXC), d.Ly, 1), th, sm, st>>>(
                 d, (const C*)pl.twz, sys, nsys, in_count, in_off, out_count, out_off, src_sel, dst_sel);
         } else {
-            smem_attr((const void*)k_fftz_green<T, CONJ, F>, sm);
-            k_fftz_green<T, CONJ, F><<<dim3(cdiv(d.Lx, TX), d.Ly, nsys), th, sm, st>>>(
+            smem_attr((const void*)k_fftz_green<T, CONJ>, sm);
+            k_fftz_green<T, CONJ><<<dim3(cdiv(d.Lx, TX), d.Ly, nsys), th, sm, st>>>(
                 d, pl.pz, (const C*)pl.twz, sys, TX, in_count, in_off, out_count, out_off, src_sel, dst_sel);
         }
         }

@@ -104,16 +104,8 @@ __device__ __forceinline__ void cp_async_elem(C* smem_dst, const C* gmem_src) {
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem_src));
 }
-__device__ __forceinline__ void cp_async_4(int* smem_dst, const int* gmem_src) {
-    const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem_src));
-}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-// wait until at most N of the most recently committed groups are still in flight
-template <int N> __device__ __forceinline__ void cp_async_wait_group() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
 
 // Element i of a fixed white field, uniform in (-1, 1) and never zero (SplitMix64's output function,
 // Steele, Lea and Flood 2014).

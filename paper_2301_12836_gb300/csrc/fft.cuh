@@ -176,10 +176,9 @@ template <int S> __device__ __forceinline__ void bfly5(fxc* v) {
     v[2] = fx_addi<S>(m2, n2); v[3] = fx_subi<S>(m2, n2);
 }
 
-// Tw: the twiddle table's entry type (C itself, or int4 for fixed point)
-template <int S, int R, typename C, typename Tw>
+template <int S, int R, typename C>
 __device__ __forceinline__ void fft_stage_r(const C* __restrict__ src, C* __restrict__ dst, int L, int Ns,
-                                            int NL, int LD, const Tw* __restrict__ tw, int tid, int nth) {
+                                            int NL, int LD, const C* __restrict__ tw, int tid, int nth) {
     const int nb = L / R;
     const int total = nb * NL;
     const int tstep = L / (Ns * R);
@@ -208,8 +207,8 @@ __device__ __forceinline__ void fft_stage_r(const C* __restrict__ src, C* __rest
 // Transform NL lines of length p.L held in buffer a (layout s[e*LD + l]); b is scratch of the
 // same size.  Returns the buffer holding the result.  The caller synchronises the block before
 // the call; the result is visible to all threads on return.  tw = exp(-2 pi i k / L), k < L.
-template <int S, typename C, typename Tw>
-__device__ C* fft_smem(C* a, C* b, const FftPlan& p, int NL, int LD, const Tw* __restrict__ tw, int tid, int nth) {
+template <int S, typename C>
+__device__ C* fft_smem(C* a, C* b, const FftPlan& p, int NL, int LD, const C* __restrict__ tw, int tid, int nth) {
     int Ns = 1;
     for (int s = 0; s < p.nst; ++s) {
         const int R = p.radix[s];

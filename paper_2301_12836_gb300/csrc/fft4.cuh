@@ -1,12 +1,10 @@
-// fft4.cuh - compile-time two-step ("four-step") FFT of lines held in shared memory.
+// fft4.cuh - compile-time two-step ("four-step") FFT.
 //
 // A line of length L = A * B is transformed as
 //   Y[t][k1] = W_L^(t k1) * sum_a x[t + B a] W_A^(a k1)      (B DFTs of length A, then twiddles)
 //   X[k1 + A k2] = sum_t Y[t][k1] W_B^(t k2)                  (A DFTs of length B)
-// with every short DFT held in registers.  Each of the two steps reads its inputs from shared
-// memory into registers, synchronises, and writes its outputs back in place, so one buffer of
-// L * LD elements suffices.  A tile of NL lines is transformed by exactly NL * min(A, B)
-// threads: thread tid works on line tid % NL.  Line l, element e sits at s[e * LD + l].
+// with every short DFT held in registers and one exchange through shared memory between the steps.  A
+// tile of NL lines is transformed by NL * min(A, B) threads: thread tid works on line tid % NL.
 #pragma once
 #include "fft.cuh"
 #include <type_traits>
@@ -254,55 +252,6 @@ template <int A, int B> struct FourStep {
     static constexpr int I2 = A / TPL;          // step-2 DFTs per thread
 };
 
-// In-place FFT (sign S) of NL lines; called by exactly NL * TPL threads, tid < NL * TPL.
-// The caller synchronises before (input written) and gets the result after the final barrier.
-// Zero padding and cropping are pruned at compile time: elements e >= NZ * B of a line are known
-// to be zero (each step-1 DFT has at most NZ nonzero inputs), and only outputs k < NO * A are
-// wanted (each step-2 DFT produces its first NO outputs; the others are left unwritten).
-template <int A, int B, int S, int NZ = A, int NO = B, typename C, typename Tw>
-__device__ __forceinline__ void fft4_smem(C* s, int NL, int LD, const Tw* __restrict__ tw, int tid) {
-    typedef FourStep<A, B> F;
-    const int l = tid % NL;
-    const int q = tid / NL;
-    C v[F::I1][A];
-#pragma unroll
-    for (int i = 0; i < F::I1; ++i) {
-        const int t = q + F::TPL * i;
-#pragma unroll
-        for (int a = 0; a < A; ++a) v[i][a] = a < NZ ? s[(t + B * a) * LD + l] : czero<C>();
-        dft_reg_p<A, S, NZ, A>(v[i]);
-        tw_row<S, A * B, A>(v[i], tw, t);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < F::I1; ++i) {
-        const int t = q + F::TPL * i;
-#pragma unroll
-        for (int k1 = 0; k1 < A; ++k1) s[(t * A + k1) * LD + l] = v[i][k1];
-    }
-    __syncthreads();
-    C w2[F::I2][B];
-#pragma unroll
-    for (int i = 0; i < F::I2; ++i) {
-        const int k1 = q + F::TPL * i;
-#pragma unroll
-        for (int t = 0; t < B; ++t) w2[i][t] = s[(t * A + k1) * LD + l];
-        dft_reg_p<B, S, B, NO>(w2[i]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < F::I2; ++i) {
-        const int k1 = q + F::TPL * i;
-#pragma unroll
-        for (int k2 = 0; k2 < NO; ++k2) s[(k1 + A * k2) * LD + l] = w2[i][k2];
-    }
-    __syncthreads();
-}
-
-}  // namespace lsm
-
-namespace lsm {
-
 // Row stride (in elements) of the step-1 intermediate Y[t][k1] of fft4_io.  Threads of a warp
 // write Y for consecutive t (groups of NL lanes) and read it back for consecutive k1; the skew
 // PAD makes each group start on the banks where the previous one ended, so both accesses cost
@@ -374,9 +323,9 @@ __device__ __forceinline__ void fft4_run(C (&v)[FourStep<A, B>::I1][A], C* s, co
 // (IN_SMEM: it reads the buffer s itself, so a barrier separates those reads from the first
 // write into s); st(l, k, v) receives output k of line l (OUT_SMEM: it writes s, so a barrier
 // separates the last reads of s from those writes).  Called by exactly NL * TPL threads.  The
-// intermediate occupies B * fft4_ystride<A, C>(NL) elements of s.  As in fft4_smem, inputs
-// e >= NZ * B are known to be zero (ld is not called for them) and only outputs k < NO * A are
-// produced (st is not called for the others).
+// intermediate occupies B * fft4_ystride<A, C>(NL) elements of s.  Zero padding and cropping are
+// pruned at compile time: inputs e >= NZ * B are known to be zero (ld is not called for them) and only
+// outputs k < NO * A are produced (st is not called for the others).
 template <int A, int B, int S, bool IN_SMEM, bool OUT_SMEM, int NL, int NZ = A, int NO = B, typename C, typename Tw, class Ld,
           class St>
 __device__ __forceinline__ void fft4_io(C* s, const Tw* __restrict__ tw, int tid, Ld ld, St st) {
