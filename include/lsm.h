@@ -176,6 +176,11 @@ lsm_status lsm_source_moments(lsm_t h, int nm, const double *M, const double xs[
 /*
  * One application of the LS operator (Eqs. 19-21): Au = A u in FP64.
  *   u, Au  device complex128, 3 * nz*ny*nx; u != Au required (no aliasing).
+ * The transforms of this and every other FP64 apply run on 64-bit integers,
+ * scaled line by line, between FP64 arrays: rounding errors are those of FP64
+ * FFTs or smaller, relative to a line's (in the z pass a column's) largest
+ * value.  Exact zeros stay zero, underflow is gradual, and an infinity or a
+ * NaN anywhere in u makes all of Au NaN.
  */
 lsm_status lsm_apply(lsm_t h, const void *u, void *Au);
 
@@ -218,8 +223,8 @@ lsm_status lsm_adjoint(lsm_t h, const void *v, void *AHv);
  *           none), on exit the solution (the last iterate on LSM_ERR_NOCONV)
  *   iters   host int* or NULL: BiCGSTAB iterations (mixed: total inner iterations)
  *   relres  host double* or NULL: the true residual ||b - A x|| / ||b|| at exit, from an
- *           FP64 apply (LSM_FP64) or the mixed mode's residual apply (double-float by
- *           default, see lsm_opts.residual), not the recursively updated one
+ *           FP64 apply (LSM_FP64) or the mixed mode's residual apply (FP64 by default,
+ *           see lsm_opts.residual), not the recursively updated one
  * Synchronises the handle's stream.
  */
 lsm_status lsm_solve(lsm_t h, const void *b, void *x, int *iters, double *relres);
@@ -327,24 +332,27 @@ long long lsm_launch_count(lsm_t h);
  * epilogue: 0 = compile-time two-step FFT where the line length allows it
  * (16..512), 1 = runtime mixed-radix Stockham engine, 2 = the same with half
  * its tile; v[3] z pass with the Green multiply: 0..2 as above (0 is the
- * register-resident kernel in FP32), 3 = the shared-memory two-step kernel.
- * Every variant computes the same operator.  precision: LSM_FP64 (the FP64
- * applies) or LSM_MIXED (the FP32 applies of a mixed handle).  The schedule
- * belongs to the medium (all handles sharing it); setting one drops the
- * captured iteration graphs.  LSM_ERR_ARG for an invalid variant.
+ * register-resident kernel in FP32), 3 = the shared-memory two-step kernel
+ * (FP64 applies have one two-step z kernel: 3 runs 0).  Where the tile of
+ * variant 1 is already the smallest (the FP64 z pass of lines longer than 128
+ * points), 2 runs 1.  Every variant computes the same operator.
+ * precision: LSM_FP64 (the FP64 applies) or LSM_MIXED (the FP32 applies of a
+ * mixed handle).  The schedule belongs to the medium (all handles sharing it);
+ * setting one drops the captured iteration graphs.  LSM_ERR_ARG for an invalid
+ * variant.
  */
 lsm_status lsm_set_schedule(lsm_t h, int precision, const int v[6]);
 lsm_status lsm_get_schedule(lsm_t h, int precision, int v[6]);
 
 /*
  * The project's tuner: times `reps` batched applies (1..100) of nsys systems
- * (1..64, the batch size the solves will use) under every variant set, per
- * precision the handle runs, with CUDA events around each stage, and keeps for
- * every stage the fastest variant.  The chosen schedules are returned in v64
- * and v32 (host int[6] each, may be NULL; v32 is all 0 for an LSM_FP64
- * handle).  Sizes the solver workspace for nsys systems and allocates 1 + nsys
- * 3N complex128 buffers for the duration; resets the stage timer's totals;
- * synchronises the stream.
+ * (1..64, the batch size the solves will use) of a white field under every
+ * variant set, per precision the handle runs, with CUDA events around each
+ * stage, and keeps for every stage the fastest variant.  The chosen schedules
+ * are returned in v64 and v32 (host int[6] each, may be NULL; v32 is all 0 for
+ * an LSM_FP64 handle).  Sizes the solver workspace for nsys systems and
+ * allocates 1 + nsys 3N complex128 buffers for the duration; resets the stage
+ * timer's totals; synchronises the stream.
  */
 lsm_status lsm_autotune(lsm_t h, int nsys, int reps, int v64[6], int v32[6]);
 

@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(3 * TX * 32) kg_fftz_green_fx(Dims d, FxPlan p
 // stored as their first half 0 .. n, n = L / 2; outputs 0 .. n in place.  Component c of the six
 // (blockIdx.z) is odd when bit c of `odd` is set.  Line i of outer group o starts at o os + i ls, its
 // elements es apart; ROWS: es = 1, loads and stores run along the line.  Outputs that vanish by
-// symmetry come out as exact zeros (fx_to_odd).
+// symmetry come out as zero or a few units: v and -v round to opposite values but for ties.
 struct SymArgs {
     long long cs, os, ls, es;
     int nlines, odd;
@@ -297,14 +297,14 @@ __global__ void __launch_bounds__(NL * 48) kg_sym_fx(FxPlan p, FxTables T, SymAr
             const FxUnit un(sk.unit(p.fxbits) + (DYN ? s_sum[k] : esum), sk.bad, s_mag[k] == 0);
             for (int e = threadIdx.x; e <= n; e += blockDim.x) {
                 const fxc v = r[e * LD + k];
-                tile[k * a.ls + e] = fx_to_odd(v, un);
+                tile[k * a.ls + e] = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
             }
         }
     } else if (l < live) {
         const FxUnit un(sc.unit(p.fxbits) + esum, sc.bad, s_mag[l] == 0);
         for (int e = g; e <= n; e += m) {
             const fxc v = r[e * LD + l];
-            tile[l * a.ls + e * a.es] = fx_to_odd(v, un);
+            tile[l * a.ls + e * a.es] = un.odd ? fx_to_odd(v, un) : fx_to(v, un);
         }
     }
 }
