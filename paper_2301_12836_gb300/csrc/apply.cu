@@ -1535,16 +1535,21 @@ static inline int fxg_width(int L, int per, int most, size_t cap, int v) {
     if (v == 2 && w > 2) w /= 2;
     return w;
 }
-// Call fn with the width and the plan's kind as constants: 8 or 4 lines, or 2 for the half tile of lines
-// too long for 8, which are all dynamic ones; z passes 4 columns or 2, dynamic plans (L > 128) 2.
-template <typename Fn> static void with_tile(int w, const FxPlan& p, Fn&& fn) {
+// Call fn with the width and the plan's kind as constants: static plans (L <= 256) 8 lines, dynamic ones 8
+// or 4, and the half of either where the schedule may ask for it (HALF).  z: 4 columns or 2, dynamic
+// plans (L > 128) 2.
+template <bool HALF, typename Fn> static void with_tile(int w, const FxPlan& p, Fn&& fn) {
     using std::integral_constant;
-    if (!p.fxdyn) {
-        if (w == 8) fn(integral_constant<int, 8>(), std::false_type());
-        else fn(integral_constant<int, 4>(), std::false_type());
-    } else if (w == 8) fn(integral_constant<int, 8>(), std::true_type());
-    else if (w == 4) fn(integral_constant<int, 4>(), std::true_type());
-    else fn(integral_constant<int, 2>(), std::true_type());
+    if (p.fxdyn) {
+        if constexpr (HALF)
+            if (w == 2) return fn(integral_constant<int, 2>(), std::true_type());
+        if (w == 8) fn(integral_constant<int, 8>(), std::true_type());
+        else fn(integral_constant<int, 4>(), std::true_type());
+    } else {
+        if constexpr (HALF)
+            if (w == 4) return fn(integral_constant<int, 4>(), std::false_type());
+        fn(integral_constant<int, 8>(), std::false_type());
+    }
 }
 template <typename Fn> static void with_ztile(int w, const FxPlan& p, Fn&& fn) {
     using std::integral_constant;
@@ -1557,7 +1562,7 @@ template <typename Fn> static void with_ztile(int w, const FxPlan& p, Fn&& fn) {
 template <int DIR, bool OUT>
 static void launch_rows_fxg(const Dims& d, const ApplySys<double>* sys, int nsys, const Plans& pl, int src_sel, int dst_sel,
                             long long nrows, int in_count, int in_off, int out_count, int out_off, cudaStream_t st, int v) {
-    with_tile(fxg_width(d.Lx, 1, 8, SMEM_CAP, v), pl.px, [&](auto w, auto dyn) {
+    with_tile<true>(fxg_width(d.Lx, 1, 8, SMEM_CAP, v), pl.px, [&](auto w, auto dyn) {
         constexpr int NL = decltype(w)::value;
         constexpr bool DYN = decltype(dyn)::value;
         const size_t sm = 2 * (size_t)d.Lx * (NL + 1) * sizeof(fxc);
@@ -1684,7 +1689,7 @@ static void launch_strided(int L, const FxPlan& p, const void* tw, const Plans& 
                 k4_strided_fx<DIR, A, B, TXC><<<dim3(cdiv(a.nlines, TXC), outer, a.ncomp * nsys), TXC * F::TPL, sm, st>>>(
                     fx_twostep(pl, axis, L), a, sys, fx_bits(L, a.in_count, DIR < 0 ? A / 2 + 1 : A, B));
             } else {
-                with_tile(fxg_width(L, 1, 8, SMEM_CAP, v), p, [&](auto w, auto dyn) {
+                with_tile<true>(fxg_width(L, 1, 8, SMEM_CAP, v), p, [&](auto w, auto dyn) {
                     constexpr int NL = decltype(w)::value;
                     constexpr bool DYN = decltype(dyn)::value;
                     const size_t sm = 2 * (size_t)L * NL * sizeof(fxc);
@@ -2192,7 +2197,7 @@ cudaError_t launch_octant_fft(const Dims& d, const Plans& pl, double2* buf, cuda
         if (a == 0) { s.ls = sx; s.es = 1; s.os = 0; s.nlines = (int)(sy * sz); }
         else if (a == 1) { s.ls = 1; s.es = sx; s.os = sx * sy; s.nlines = (int)sx; outer = (int)sz; }
         else { s.ls = 1; s.es = sx * sy; s.os = 0; s.nlines = (int)(sx * sy); }
-        with_tile(fxg_width(p[a]->L, 1, 8, SMEM_CAP, 0), *p[a], [&](auto w, auto dyn) {
+        with_tile<false>(fxg_width(p[a]->L, 1, 8, SMEM_CAP, 0), *p[a], [&](auto w, auto dyn) {
             constexpr int NL = decltype(w)::value;
             constexpr bool DYN = decltype(dyn)::value;
             const int m = fxg_groups(*p[a], 64 / NL, NL < 4 ? 48 : 192 / NL);
