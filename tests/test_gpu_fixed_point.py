@@ -20,6 +20,7 @@ pytestmark = pytest.mark.gpu
 
 W = 2 * np.pi * 9.0
 # every compile-time line length (16 .. 512) on every axis, beside generic ones
+# (512, that is sides of 256, in test_gpu_fixed_point_long.py)
 GRIDS = [(8, 16, 32), (32, 8, 16), (16, 32, 8), (64, 9, 8), (12, 64, 10), (8, 10, 64), (128, 8, 9), (9, 128, 8), (8, 9, 128)]
 
 
